@@ -32,6 +32,7 @@ namespace {
 using namespace upd;
 
 constexpr int kBThreads = 128;
+constexpr int kBBlocksPerSM = 4;          // as the single contexts' phase kernel
 constexpr int kMaxRefs = 256;
 constexpr int kViewWords = (int)(sizeof(ViewConst) / sizeof(float));   // a view table entry in 4-byte words
 static_assert(sizeof(ViewConst) % sizeof(float) == 0, "view table entries are whole words");
@@ -95,8 +96,9 @@ struct TileShape {
 };
 
 template <bool kHalf, int TW, int WC, int kMode>
-__global__ void __launch_bounds__(kBThreads, 3) batch_phase_kernel(const __grid_constant__ BatchArgs b) {
+__global__ void __launch_bounds__(kBThreads, kBBlocksPerSM) batch_phase_kernel(const __grid_constant__ BatchArgs b) {
   __shared__ RefArgs ra;
+  __shared__ WinShared ws;
   __shared__ int cur_ref, item_slot;
   using T = TileShape<TW, WC>;
   int npairs = 0;
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(kBThreads, 3) batch_phase_kernel(const __grid_
     const int x = tx * TW + 2 * T::col(threadIdx.x) + ((y + b.color) & 1);
     if (x < ra.W && y < ra.H) {
       PixelArrays sm;
-      update_pixel<kHalf, kMode>(ra, sm, x, y, &npairs);
+      update_pixel<kHalf, kMode>(ra, sm, x, y, &npairs, ws.q + threadIdx.x);
     }
   }
   const int tot = __reduce_add_sync(0xffffffffu, npairs);
@@ -135,8 +137,9 @@ __global__ void __launch_bounds__(kBThreads, 3) batch_phase_kernel(const __grid_
 
 // random initialisation of every pixel of every reference: 16 x 8 pixel tiles
 template <bool kHalf, bool kTex>
-__global__ void __launch_bounds__(kBThreads) batch_init_kernel(const __grid_constant__ BatchArgs b) {
+__global__ void __launch_bounds__(kBThreads, kBBlocksPerSM) batch_init_kernel(const __grid_constant__ BatchArgs b) {
   __shared__ RefArgs ra;
+  __shared__ WinShared ws;
   __shared__ int cur_ref, item_slot;
   int npairs = 0;
   if (threadIdx.x == 0) cur_ref = -1;
@@ -158,7 +161,7 @@ __global__ void __launch_bounds__(kBThreads) batch_init_kernel(const __grid_cons
     const int x = tx * 16 + (threadIdx.x & 15), y = ty * 8 + (threadIdx.x >> 4);
     if (x < ra.W && y < ra.H) {
       PixelArrays sm;
-      init_pixel<kHalf, kTex>(ra, sm, x, y, &npairs);
+      init_pixel<kHalf, kTex>(ra, sm, x, y, &npairs, ws.q + threadIdx.x);
     }
   }
   const int tot = __reduce_add_sync(0xffffffffu, npairs);
@@ -548,7 +551,7 @@ AMH_API int amh_batch_create(amh_batch** out, const amh_params* p, int32_t n_vie
   int dev = 0, sms = 0;
   CB(cudaGetDevice(&dev));
   CB(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  b->grid_blocks = sms * 3;   // persistent: three 128-thread blocks per SM
+  b->grid_blocks = sms * kBBlocksPerSM;
   CB(cudaStreamSynchronize(b->stream));
 #undef CB
   *out = b;

@@ -177,7 +177,12 @@ __device__ __forceinline__ float3 ref_ray(const float* Ki, float x, float y) {
   return make_float3(fmaf(Ki[0], x, fmaf(Ki[1], y, Ki[2])), fmaf(Ki[3], x, fmaf(Ki[4], y, Ki[5])),
                      fmaf(Ki[6], x, fmaf(Ki[7], y, Ki[8])));
 }
-__device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// The order of the two fused steps is written out, so that every kernel that
+// updates a pixel rounds alike (the compiler may otherwise fuse either product).
+__device__ __forceinline__ float dot3(float3 a, float3 b) { return fmaf(a.z, b.z, fmaf(a.x, b.x, __fmul_rn(a.y, b.y))); }
+__device__ __forceinline__ float dot3_xfirst(float3 a, float3 b) {
+  return fmaf(a.z, b.z, fmaf(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
 
 __device__ __forceinline__ float3 face_camera(float3 n, float3 ray) {
   if (!(dot3(n, ray) < 0.f)) { n.x = -n.x; n.y = -n.y; n.z = -n.z; }
@@ -194,15 +199,18 @@ __device__ __forceinline__ float3 normal_from_uniforms(float u1, float u2) {
 
 // The cost needs c = K_ref^-T n / d (Sec. 2) with d = -D (n . ray) the plane
 // offset, and 1 / D (the window centre's image, see ViewConst); the plane is
-// usable when it faces the pixel (d > 0) at D > 0.  c.w = 1 / D.
+// usable when it faces the pixel (d > 0) at D > 0.  c.w = 1 / D.  The refinement
+// candidates have always been rounded x first (kXFirst); every other plane y
+// first.
+template <bool kXFirst = false>
 __device__ __forceinline__ bool plane_c(const float* Ki, float4 pl, float3 ray, float4* c) {
   const float3 n = make_float3(pl.x, pl.y, pl.z);
-  const float d = -pl.w * dot3(n, ray);
+  const float d = -pl.w * (kXFirst ? dot3_xfirst(n, ray) : dot3(n, ray));
   const bool ok = (pl.w > 0.f) && (d > 0.f) && isfinite(d);
   const float id = ok ? 1.f / d : 0.f;
-  *c = make_float4((Ki[0] * n.x + Ki[3] * n.y + Ki[6] * n.z) * id,
-                   (Ki[1] * n.x + Ki[4] * n.y + Ki[7] * n.z) * id,
-                   (Ki[2] * n.x + Ki[5] * n.y + Ki[8] * n.z) * id, ok ? 1.f / pl.w : 0.f);
+  *c = make_float4(dot3(make_float3(Ki[0], Ki[3], Ki[6]), n) * id,
+                   dot3(make_float3(Ki[1], Ki[4], Ki[7]), n) * id,
+                   dot3(make_float3(Ki[2], Ki[5], Ki[8]), n) * id, ok ? 1.f / pl.w : 0.f);
   return ok;
 }
 

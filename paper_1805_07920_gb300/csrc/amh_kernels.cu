@@ -16,7 +16,12 @@ using namespace upd;
 
 constexpr int kTile = 16;
 constexpr int kThreads = 128;
-constexpr int kPhaseBlocksPerSM = 3;          // 168 registers per thread
+// 128 registers per thread; the window weights are 36 KB of shared memory per
+// block, so 4 blocks leave about 100 KB of L1.  3200 x 2112, 10 sources, six
+// iterations: 3 blocks 171 ms, 4: 165.5, 5 (96 registers): 165.4, and 5 lost
+// 2 - 5 % on the smaller images (all before the rows ran in two passes, see
+// ncc_window).  The staged sweep's boxes allow 3.
+constexpr int kPhaseBlocksPerSM = 4, kStagedBlocksPerSM = 3;
 
 // npairs: evaluations of this thread, plus 2^16 for each one sampled from a
 // shared-memory box (fewer than 2^11 per thread and launch); the two totals
@@ -30,8 +35,9 @@ __device__ __forceinline__ void count_pairs(const PhaseArgs& a, int npairs) {
 }
 
 template <bool kHalf, int kMode>
-__global__ void __launch_bounds__(kThreads, kPhaseBlocksPerSM) phase_kernel(const __grid_constant__ PhaseArgs a) {
+__global__ void __launch_bounds__(kThreads, (kMode & kStage) ? kStagedBlocksPerSM : kPhaseBlocksPerSM) phase_kernel(const __grid_constant__ PhaseArgs a) {
   PixelArrays sm;
+  __shared__ WinShared ws;
   const int tid = threadIdx.x;
   int npairs = 0;
   if constexpr ((kMode & kStage) != 0) {
@@ -44,44 +50,50 @@ __global__ void __launch_bounds__(kThreads, kPhaseBlocksPerSM) phase_kernel(cons
     const int x = blockIdx.x * kTile + 2 * (4 * (q & 1) + (lane & 3)) + ((y + a.color) & 1);
     // the whole block takes part in the staged sweep, pixels outside the image too
     __shared__ StageShared ss;
-    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, &ss, x < a.W && y < a.H);
+    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, &ss, x < a.W && y < a.H);
   } else {
     const int y = blockIdx.y * kTile + (tid >> 3);
     const int x = blockIdx.x * kTile + 2 * (tid & 7) + ((y + a.color) & 1);
-    if (x < a.W && y < a.H) update_pixel<kHalf, kMode>(a, sm, x, y, &npairs);
+    if (x < a.W && y < a.H) update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid);
   }
   count_pairs(a, npairs);
 }
 
 // Random initialisation: one thread per pixel over the whole image.
 template <bool kHalf, bool kTex>
-__global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ PhaseArgs a) {
+__global__ void __launch_bounds__(kThreads, kPhaseBlocksPerSM) init_kernel(const __grid_constant__ PhaseArgs a) {
   PixelArrays sm;
+  __shared__ WinShared ws;
   const int x = blockIdx.x * kTile + (threadIdx.x & 15), y = blockIdx.y * 8 + (threadIdx.x >> 4);
   int npairs = 0;
-  if (x < a.W && y < a.H) init_pixel<kHalf, kTex>(a, sm, x, y, &npairs);
+  if (x < a.W && y < a.H) init_pixel<kHalf, kTex>(a, sm, x, y, &npairs, ws.q + threadIdx.x);
   count_pairs(a, npairs);
 }
 
 
 }  // namespace
 
-// Both kernels use no shared memory: ask for the largest L1 (texture cache).
-// The preference is per device, so it is set once for each device that
-// launches the kernel.
+// Ask for the smallest shared-memory carve-out that holds `blocks` blocks of
+// `smem` bytes (and the 1 KB each that the system keeps): the rest of the
+// unified L1 is texture and local-memory cache.  The preference is per device,
+// so it is set once for each device that launches the kernel.
 template <typename K>
-void prefer_l1(K kernel, std::once_flag* once) {
+void prefer_carveout(K kernel, int blocks, int smem, std::once_flag* once) {
   int dev = 0;
   cudaGetDevice(&dev);
-  std::call_once(once[dev & 63], [kernel] {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  std::call_once(once[dev & 63], [=] {
+    int smem_sm = 0;
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const int need = blocks * (smem + 1024);
+    const int pct = smem_sm > 0 ? std::min(100, (100 * need + smem_sm - 1) / smem_sm) : 100;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   });
 }
 
 template <bool kHalf, bool kTex>
 int launch_init_t(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
-  prefer_l1(init_kernel<kHalf, kTex>, once);
+  prefer_carveout(init_kernel<kHalf, kTex>, kPhaseBlocksPerSM, (int)sizeof(WinShared), once);
   dim3 grid((a.W + kTile - 1) / kTile, (a.H + 7) / 8);
   init_kernel<kHalf, kTex><<<grid, kThreads, 0, s>>>(a);
   return (int)cudaGetLastError();
@@ -96,22 +108,9 @@ int launch_init(const PhaseArgs& a, cudaStream_t s) {
 template <bool kHalf, int kMode>
 int launch_phase_t(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
-  if ((kMode & kStage) == 0) {
-    prefer_l1(phase_kernel<kHalf, kMode>, once);
-  } else {
-    // the smallest carve-out that holds the staged blocks' shared memory: the
-    // rest of the unified L1 stays texture and local-memory cache
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::call_once(once[dev & 63], [] {
-      int d = 0, smem_sm = 0;
-      cudaGetDevice(&d);
-      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, d);
-      const int need = kPhaseBlocksPerSM * (int)(sizeof(StageShared) + 1024);
-      const int pct = smem_sm > 0 ? std::min(100, (100 * need + smem_sm - 1) / smem_sm) : 100;
-      cudaFuncSetAttribute(phase_kernel<kHalf, kMode>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-    });
-  }
+  constexpr bool kStaged = (kMode & kStage) != 0;
+  prefer_carveout(phase_kernel<kHalf, kMode>, kStaged ? kStagedBlocksPerSM : kPhaseBlocksPerSM,
+                  (int)(sizeof(WinShared) + (kStaged ? sizeof(StageShared) : 0)), once);
   dim3 grid((a.W + kTile - 1) / kTile, (a.H + kTile - 1) / kTile);
   phase_kernel<kHalf, kMode><<<grid, kThreads, 0, s>>>(a);
   return (int)cudaGetLastError();

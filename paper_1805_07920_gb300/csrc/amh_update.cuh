@@ -7,10 +7,11 @@
 // Work mapping: one thread per reference pixel; a warp updates 32 pixels of
 // one colour of a compact tile, so the lanes of every texture gather sample
 // neighbouring windows of the same source view.  Every (hypothesis, view)
-// loop runs with a warp-uniform view index (uniform texture handle).  Each
-// thread keeps its 36 bilateral weights in registers and its cost matrix and
-// view weights in local memory (L1); no shared memory is needed, so the whole
-// L1 serves the texture gathers.
+// loop runs with a warp-uniform view index (uniform texture handle).  The 36
+// bilateral weights of a pixel sit in shared memory (72 floats read once per
+// evaluation, conflict-free 16-byte loads): in registers they held the kernel
+// at 168 registers and 12 warps per SM, here 128 and 16.  The cost matrix and
+// the view weights are in local memory (L1).
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -56,12 +57,27 @@ static_assert(acp_other_colour(), "propagation candidates lie on the other colou
 // {-5,-3,-1,1,3,5}^2 clamped to the image; w = exp(-|I - I_c| / (2 sigma_I^2)
 // - |dx| / (2 sigma_x^2)); the values centred on their weighted mean so that
 // cov(r, s) = sum w r^ s / sum w.
-// Stored as lane pairs (samples 2m, 2m + 1) for the packed moment updates.
+// The weights sit in shared memory as lane pairs (samples 2m, 2m + 1) for the
+// packed moment updates: (w, w', w r, w' r') of pair m at q[m * kStep], kStep
+// pixels side by side.
+constexpr int kWinPairs = kWinS / 2;
+template <int kStep>
 struct RefWin {
-  f2 w2[kWinS / 2];
-  f2 wr2[kWinS / 2];
+  float4* q;
   float inv_sw, sum_wr, var_r;
+  __device__ __forceinline__ void pair(int m, f2& w, f2& wr) const {
+    const float4 v = q[m * kStep];
+    w = pack2(v.x, v.y);
+    wr = pack2(v.z, v.w);
+  }
 };
+constexpr int kBlockPixels = 128;         // pixels of a block, one per thread
+using PixelWin = RefWin<kBlockPixels>;
+struct WinShared {
+  float4 q[kWinPairs * kBlockPixels];
+};
+constexpr int kTeamPixels = 32;           // pixels of a team, one per lane
+using TeamWin = RefWin<kTeamPixels>;
 static_assert(kWinS % 2 == 0 && kWinN % 2 == 0, "window samples are processed in pairs along a row");
 
 // intensity of reference pixel i (uint8 or FP16 images)
@@ -76,8 +92,8 @@ __device__ __forceinline__ float ref_at(const A& a, size_t i) {
 template <bool kHalf>
 __host__ __device__ constexpr float tex_scale() { return kHalf ? 1.f : 255.f; }
 
-template <bool kHalf, class A>
-__device__ __forceinline__ void load_ref_window(const A& a, int x, int y, RefWin& rw) {
+template <bool kHalf, int kStep, class A>
+__device__ __forceinline__ void load_ref_window(const A& a, int x, int y, RefWin<kStep>& rw) {
   const float Ic = ref_at<kHalf, A>(a, (size_t)y * a.W + x);
   // w = exp(-e) relative to the largest weight: the statistics of Eq. (8) are
   // ratios of weighted sums, so the common factor cancels, and no weight
@@ -112,13 +128,12 @@ __device__ __forceinline__ void load_ref_window(const A& a, int x, int y, RefWin
     const float rc = rv[k] - mr;
     const float wr = wv[k] * rc;
     wrv[k] = wr;
-    swr += wr;
+    swr = __fadd_rn(swr, wr);
     s2 = fmaf(wr, rc, s2);
   }
 #pragma unroll
   for (int m = 0; m < kWinS / 2; m++) {
-    rw.w2[m] = pack2(wv[2 * m], wv[2 * m + 1]);
-    rw.wr2[m] = pack2(wrv[2 * m], wrv[2 * m + 1]);
+    rw.q[m * kStep] = make_float4(wv[2 * m], wv[2 * m + 1], wrv[2 * m], wrv[2 * m + 1]);
   }
   rw.inv_sw = inv;
   rw.sum_wr = swr;
@@ -222,12 +237,49 @@ __device__ __forceinline__ f2 floor2_bits(f2 x, uint32_t& bx, uint32_t& by) {
   return sub2(t, M);
 }
 
+// One texture fetch of a window sample: the 2 x 2 texels at floored position
+// (x, y) (kFetchGather), or the filtered value (kFetchFilter).  Volatile, so
+// that a group's fetches all stand before the arithmetic on their results.
+__device__ __forceinline__ float4 tex_gather(cudaTextureObject_t t, float x, float y) {
+  float4 g;
+  asm volatile("tld4.r.2d.v4.f32.f32 {%0, %1, %2, %3}, [%4, {%5, %6}];"
+               : "=f"(g.x), "=f"(g.y), "=f"(g.z), "=f"(g.w)
+               : "l"(t), "f"(x), "f"(y));
+  return g;
+}
+__device__ __forceinline__ float tex_filter(cudaTextureObject_t t, float x, float y) {
+  float4 v;
+  asm volatile("tex.2d.v4.f32.f32 {%0, %1, %2, %3}, [%4, {%5, %6}];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(t), "f"(x), "f"(y));
+  return v.x;
+}
+
+// A row of window samples in flight: the fetched texels (or, in .x, the
+// filtered value) and the fractions.
+struct RowFetch {
+  float4 g[kWinN];
+  f2 fr[kWinN];
+};
+
 // The 36 samples of one pair and the NCC of Eq. (8).  kFetchBox: box_cells
 // is the box's cell array and box_adj its box_adjust(), so that the cell of
 // a sample whose floored positions have the bits (bx, by) is
 // by kBoxW + bx - box_adj.
-template <bool kHalf, int kFetch>
-__device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& G, const RefWin& rw,
+//
+// What bounds it: alone, one warp takes 1450 clocks for the 36 gathers; the
+// texture unit saturates at 1.04 - 1.10 T samples/s from 8 warps per SM on
+// (measured with this function in a loop).  In the update it competes with the
+// instruction cache: with all six rows unrolled the three inlined copies are
+// ~45 KB and "no instruction" was 12 % of the warps' time at 16 warps per SM.
+// So the rows run in two passes of kRowGroup = 3, 18 fetches in flight before
+// the first is used (about 110 of the 128 registers).  1600 x 1056, 10 sources,
+// five iterations with the proposal: 6 rows unrolled 35.5 ms, 3: 33.5, 2: 34.0,
+// 1: 35.2 (12 warps per SM, weights in registers, everything unrolled: 38.0).
+constexpr int kRowGroup = 3;
+static_assert(kWinN % kRowGroup == 0, "the rows of a window are processed in whole groups");
+template <bool kHalf, int kFetch, class Win>
+__device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& G, const Win& rw,
                                             const void* box_cells = nullptr, uint32_t box_adj = 0u) {
   const float H0 = G.H0, H1 = G.H1, H3 = G.H3, H4 = G.H4, H6 = G.H6, H7 = G.H7;
   const float px = G.px, py = G.py, pz = G.pz;
@@ -242,16 +294,14 @@ __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& 
   const float4* box = reinterpret_cast<const float4*>(box_cells);
   if (kFetch == kFetchBox) __builtin_assume(__isShared(box) != 0);
   const f2 cxy = pack2(cxs, cys), cz2 = pack2(czs, czs);
+  const cudaTextureObject_t tex = V.tex;
   f2 acc1 = pack2(0.f, 0.f), acc2 = pack2(0.f, 0.f), accr = pack2(0.f, 0.f);
   f2 s0p = pack2(0.f, 0.f);
-#pragma unroll
-  for (int ra = 0; ra < kWinN; ra++) {
-    const float bx = fmaf((float)ra, rxs, sx0), by = fmaf((float)ra, rys, sy0), bz = fmaf((float)ra, rzs, sz0);
+  auto issue = [&](float ra, RowFetch& F) {
+    const float bx = fmaf(ra, rxs, sx0), by = fmaf(ra, rys, sy0), bz = fmaf(ra, rzs, sz0);
     const f2 bxy = pack2(bx, by), bz2 = pack2(bz, bz);
 #pragma unroll
     for (int cb = 0; cb < kWinN; cb += 2) {
-      const int m = (ra * kWinN + cb) / 2;
-      // (x, y) of each sample in one lane pair (the gather takes them as a pair)
       const f2 qa = fma2(pack2((float)cb, (float)cb), cxy, bxy);
       const f2 qb = fma2(pack2((float)(cb + 1), (float)(cb + 1)), cxy, bxy);
       const f2 qz = fma2(pack2((float)cb, (float)(cb + 1)), cz2, bz2);
@@ -261,7 +311,6 @@ __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& 
       unpack2(qb, qxb, qyb);
       const float ia = rcp_approx(qz0), ib = rcp_approx(qz1);
       const f2 pa = pack2(qxa * ia, qya * ia), pb = pack2(qxb * ib, qyb * ib);
-      f2 sp;
       if (kFetch == kFetchFilter) {
         // the texture unit's linear filter (AMH_FLAG_TEXTURE_BILINEAR): its
         // texel centres sit at +0.5, the positions here at +1
@@ -269,48 +318,68 @@ __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& 
         float hxa, hya, hxb, hyb;
         unpack2(ha, hxa, hya);
         unpack2(hb, hxb, hyb);
-        sp = pack2(tex2D<float>(V.tex, hxa, hya), tex2D<float>(V.tex, hxb, hyb));
+        F.g[cb].x = tex_filter(tex, hxa, hya);
+        F.g[cb + 1].x = tex_filter(tex, hxb, hyb);
       } else if (kFetch == kFetchBox) {
         // cell index (floor(p) - 1 - o) from the bits of the floored
         // positions; box_adj folds in the origin and the 2^23 offsets
         uint32_t bxa, bya, bxb, byb;
         const f2 fla = floor2_bits(pa, bxa, bya), flb = floor2_bits(pb, bxb, byb);
-        const f2 fra = sub2(pa, fla), frb = sub2(pb, flb);
-        const float4 ca = box[bya * (uint32_t)kBoxW + bxa - box_adj];
-        const float4 cb4 = box[byb * (uint32_t)kBoxW + bxb - box_adj];
-        float fxa, fya, fxb, fyb;
-        unpack2(fra, fxa, fya);
-        unpack2(frb, fxb, fyb);
-        sp = pack2(fmaf(fya, fmaf(fxa, ca.w, ca.z), fmaf(fxa, ca.y, ca.x)),
-                   fmaf(fyb, fmaf(fxb, cb4.w, cb4.z), fmaf(fxb, cb4.y, cb4.x)));
+        F.fr[cb] = sub2(pa, fla);
+        F.fr[cb + 1] = sub2(pb, flb);
+        F.g[cb] = box[bya * (uint32_t)kBoxW + bxa - box_adj];
+        F.g[cb + 1] = box[byb * (uint32_t)kBoxW + bxb - box_adj];
       } else {
         const f2 fla = floor2(pa), flb = floor2(pb);
-        const f2 fra = sub2(pa, fla), frb = sub2(pb, flb);
-        float x0a, x0b, y0a, y0b, fxa, fxb, fya, fyb;
+        F.fr[cb] = sub2(pa, fla);
+        F.fr[cb + 1] = sub2(pb, flb);
+        float x0a, x0b, y0a, y0b;
         unpack2(fla, x0a, y0a);
         unpack2(flb, x0b, y0b);
-        unpack2(fra, fxa, fya);
-        unpack2(frb, fxb, fyb);
-        // texels: w (x0, y0), z (x0+1, y0), x (x0, y0+1), y (x0+1, y0+1)
-        const float4 ga = tex2Dgather<float4>(V.tex, x0a, y0a, 0);
-        const float4 gb = tex2Dgather<float4>(V.tex, x0b, y0b, 0);
-        const float ta = fmaf(fxa, ga.z - ga.w, ga.w), ba = fmaf(fxa, ga.y - ga.x, ga.x);
-        const float tb = fmaf(fxb, gb.z - gb.w, gb.w), bb = fmaf(fxb, gb.y - gb.x, gb.x);
-        sp = pack2(fmaf(fya, ba - ta, ta), fmaf(fyb, bb - tb, tb));
+        F.g[cb] = tex_gather(tex, x0a, y0a);
+        F.g[cb + 1] = tex_gather(tex, x0b, y0b);
       }
+    }
+  };
+  auto value = [&](const RowFetch& F, int cb) {
+    const float4 g = F.g[cb];
+    if (kFetch == kFetchFilter) return g.x;
+    float fx, fy;
+    unpack2(F.fr[cb], fx, fy);
+    if (kFetch == kFetchBox) return fmaf(fy, fmaf(fx, g.w, g.z), fmaf(fx, g.y, g.x));
+    // texels: w (x0, y0), z (x0+1, y0), x (x0, y0+1), y (x0+1, y0+1)
+    const float ta = fmaf(fx, g.z - g.w, g.w), ba = fmaf(fx, g.y - g.x, g.x);
+    return fmaf(fy, ba - ta, ta);
+  };
+  auto consume = [&](int ra, const RowFetch& F) {
+#pragma unroll
+    for (int cb = 0; cb < kWinN; cb += 2) {
+      const f2 sp = pack2(value(F, cb), value(F, cb + 1));
       // moments about the first sample: exact zero variance for constant
       // patches in FP32
-      if (m == 0) {
-        float s0, s1_;
+      if (cb == 0) {
+        float s0, s1_, t0, t1_;
         unpack2(sp, s0, s1_);
+        unpack2(s0p, t0, t1_);
+        s0 = ra == 0 ? s0 : t0;
         s0p = pack2(s0, s0);
       }
       const f2 sc = sub2(sp, s0p);
-      const f2 ws = mul2(rw.w2[m], sc);
+      f2 w2, wr2;
+      rw.pair(ra * (kWinN / 2) + cb / 2, w2, wr2);
+      const f2 ws = mul2(w2, sc);
       acc1 = add2(acc1, ws);
       acc2 = fma2(ws, sc, acc2);
-      accr = fma2(rw.wr2[m], sc, accr);
+      accr = fma2(wr2, sc, accr);
     }
+  };
+#pragma unroll 1
+  for (int r0 = 0; r0 < kWinN; r0 += kRowGroup) {
+    RowFetch F[kRowGroup];
+#pragma unroll
+    for (int u = 0; u < kRowGroup; u++) issue((float)(r0 + u), F[u]);
+#pragma unroll
+    for (int u = 0; u < kRowGroup; u++) consume(r0 + u, F[u]);
   }
   float m1a, m1b, m2a, m2b, mra, mrb;
   unpack2(acc1, m1a, m1b);
@@ -327,9 +396,9 @@ __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& 
   return fminf(fmaxf(1.f - cov * (S * rsqrtf(vv)), 0.f), 2.f);
 }
 
-template <bool kHalf, bool kTex = false>
+template <bool kHalf, bool kTex = false, class Win>
 __device__ __forceinline__ float ncc_cost(const ViewConst& V, float4 c, bool ok, float3 ray,
-                                          const RefWin& rw, int* evaluated) {
+                                          const Win& rw, int* evaluated) {
   if (!ok) return kWorst;
   PairGeom G;
   if (!pair_geometry(V, c, ray, G)) return kWorst;
@@ -344,7 +413,7 @@ __device__ __forceinline__ float ncc_cost(const ViewConst& V, float4 c, bool ok,
 // order of operations).
 template <bool kHalf>
 __device__ __forceinline__ float ncc_cost_boxed(const ViewConst& V, float4 c, bool ok, float3 ray,
-                                                const RefWin& rw, int* evaluated, const BoxPlace& bp,
+                                                const PixelWin& rw, int* evaluated, const BoxPlace& bp,
                                                 const SampleBox& box, uint32_t box_adj) {
   PairGeom G;
   const bool act = ok && pair_geometry(V, c, ray, G);
@@ -572,6 +641,33 @@ __device__ __forceinline__ float kbest_mean(const float* m, int N, int k) {
   return acc / (float)k;
 }
 
+// The plane pq of pixel (qx, qy) re-expressed at the pixel with the given ray:
+// its depth there and c (plane_c); false when it does not face the pixel.
+template <class A>
+__device__ __forceinline__ bool propagate(const A& a, float4 pq, int qx, int qy, float3 ray, float* Dx, float4* c) {
+  const float3 nq = make_float3(pq.x, pq.y, pq.z);
+  const float3 rq = ref_ray(a.Kinv, (float)qx, (float)qy);
+  const float d = -pq.w * dot3(nq, rq);          // plane offset, the same at q and x
+  const float den = dot3(nq, ray);
+  if (!(den < 0.f)) return false;
+  *Dx = -d / den;
+  if (!(*Dx > 0.f) || !isfinite(*Dx)) return false;
+  return plane_c(a.Kinv, make_float4(nq.x, nq.y, nq.z, *Dx), ray, c);
+}
+// The learned proposal (n, d) of pixel (x, y)'s 2 x 2 block as a plane at the
+// pixel; false when there is none that faces it.
+template <class A>
+__device__ __forceinline__ bool learned_plane(const A& a, int x, int y, float3 ray, float4* prop) {
+  *prop = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!a.prop) return false;
+  const float4 pr = a.prop[checked_index(a, (size_t)min(y / 2, a.prop_h - 1) * a.prop_w + min(x / 2, a.prop_w - 1),
+                                         (size_t)a.prop_w * a.prop_h, kBadProposal)];
+  const float den = dot3(make_float3(pr.x, pr.y, pr.z), ray);
+  const float Dx = den < 0.f ? -pr.w / den : 0.f;
+  *prop = make_float4(pr.x, pr.y, pr.z, Dx);
+  return pr.w > 0.f && Dx > 0.f && isfinite(Dx);
+}
+
 // Ablations of Sec. 4 (template bits of update_pixel): kSymmetric -- each of
 // the 8 regions is one fixed candidate, the axis neighbour at distance 1
 // (regions 0-3) or 5 (regions 4-7) up, down, left, right, instead of the
@@ -591,7 +687,7 @@ constexpr int kStage = 8;
 // ---------------------------------------------------------------------------
 template <bool kHalf, int kMode = 0, class A>
 __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x, int y,
-                                             int* npairs, StageShared* ss = nullptr, bool live = true) {
+                                             int* npairs, float4* win, StageShared* ss = nullptr, bool live = true) {
   constexpr bool kTex = (kMode & kTexture) != 0;
   constexpr bool kStaged = (kMode & kStage) != 0;
   static_assert(!(kStaged && kTex), "the staged sweep gathers; the texture-filter form does not stage");
@@ -649,23 +745,16 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
   for (int g = 0; g < kRegions; g++) {
     hD[g] = 0.f;
     if (pick[g] < 0) continue;
-    const float4 pq = a.plane[pick_index(pick[g])];
-    const float3 nq = make_float3(pq.x, pq.y, pq.z);
-    const int qx = x + (pick[g] & 255) - 32, qy = y + (pick[g] >> 8) - 32;
-    const float3 rq = ref_ray(a.Kinv, (float)qx, (float)qy);
-    const float d = -pq.w * dot3(nq, rq);          // plane offset, the same at q and x
-    const float den = dot3(nq, ray);
-    if (!(den < 0.f)) continue;
-    const float Dx = -d / den;
-    if (!(Dx > 0.f) || !isfinite(Dx)) continue;
+    float Dx;
     float4 c;
-    if (!plane_c(a.Kinv, make_float4(nq.x, nq.y, nq.z, Dx), ray, &c)) continue;
+    if (!propagate(a, a.plane[pick_index(pick[g])], x + (pick[g] & 255) - 32, y + (pick[g] >> 8) - 32, ray, &Dx, &c)) continue;
     sm.cc(g) = c;
     hD[g] = Dx;
     valid |= 1u << g;
   }
 
-  RefWin rw;
+  PixelWin rw;
+  rw.q = win;
   if (live) load_ref_window<kHalf>(a, x, y, rw);
 
   // --- Eq. (1): the 8 x N cost matrix (views outer: the 8 hypotheses of a view
@@ -797,16 +886,8 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
   // A learned proposal (n, d) of this pixel's 2 x 2 block, when present, is one
   // more candidate after the refinement ones, scored with the same weights.
   const int nc = a.t < 3 ? 1 : kMaxRefine;
-  float4 prop = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool has_prop = false;
-  if (a.prop) {
-    const float4 pr = a.prop[checked_index(a, (size_t)min(y / 2, a.prop_h - 1) * a.prop_w + min(x / 2, a.prop_w - 1),
-                                           (size_t)a.prop_w * a.prop_h, kBadProposal)];
-    const float den = pr.x * ray.x + pr.y * ray.y + pr.z * ray.z;
-    const float Dx = den < 0.f ? -pr.w / den : 0.f;
-    has_prop = pr.w > 0.f && Dx > 0.f && isfinite(Dx);
-    prop = make_float4(pr.x, pr.y, pr.z, Dx);
-  }
+  float4 prop;
+  const bool has_prop = learned_plane(a, x, y, ray, &prop);
   const int ncand = nc + (has_prop ? 1 : 0);
   // The outcome is the candidate of least cost strictly below the current
   // best (ties: the lower index).  The candidates are scored view by view:
@@ -823,7 +904,7 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
 #pragma unroll 1
   for (int ci = 0; ci < ncand; ci++) {
     float4 cc;
-    if (plane_c(a.Kinv, ci < nc ? refine_candidate(a, x, y, best, ray, ci) : prop, ray, &cc)) okm |= 1u << ci;
+    if (plane_c<true>(a.Kinv, ci < nc ? refine_candidate(a, x, y, best, ray, ci) : prop, ray, &cc)) okm |= 1u << ci;
     sm.cc(ci) = cc;
     sm.m(0, ci, N) = 0.f;
   }
@@ -868,7 +949,7 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
 // face the camera, draws (pixel, 0, 0, 0); the initial cost is the mean of the
 // k smallest per-view costs, summed in ascending order (ties: lower view).
 template <bool kHalf, bool kTex, class A>
-__device__ __forceinline__ void init_pixel(const A& a, PixelArrays& sm, int x, int y, int* npairs) {
+__device__ __forceinline__ void init_pixel(const A& a, PixelArrays& sm, int x, int y, int* npairs, float4* win) {
   const int N = a.N;
   const size_t pi = checked_index(a, state_index(x, y, a.W), state_size(a.W, a.H), kBadPixel);
   const float fx = (float)x, fy = (float)y;
@@ -878,7 +959,8 @@ __device__ __forceinline__ void init_pixel(const A& a, PixelArrays& sm, int x, i
   const float4 pl = make_float4(n.x, n.y, n.z, a.dmin + (a.dmax - a.dmin) * u01(r.x));
   float4 c;
   const bool ok = plane_c(a.Kinv, pl, ray, &c);
-  RefWin rw;
+  PixelWin rw;
+  rw.q = win;
   load_ref_window<kHalf>(a, x, y, rw);
   for (int j = 0; j < N; j++) sm.wt(j) = ncc_cost<kHalf, kTex>(a.v[j], c, ok, ray, rw, npairs);
   // mean of the k smallest per-view costs, summed in ascending order (ties:

@@ -8,6 +8,7 @@
 
 #include "amh_device.cuh"
 #include "amh_kernels.h"
+#include "amh_team.cuh"
 #include "amh_update.cuh"
 
 namespace amh {
@@ -70,6 +71,29 @@ __global__ void __launch_bounds__(kThreads, kPhaseBlocksPerSM) init_kernel(const
   count_pairs(a, npairs);
 }
 
+// Small images: a team of T warps per 16 x 4 tile (32 pixels of the colour), or
+// per 8 x 4 tile of the initialisation.
+template <int T>
+constexpr int kTeamBlocksPerSM = 16 / T;      // 16 warps, 128 registers per thread, as phase_kernel
+template <bool kHalf, bool kTex, int T>
+__global__ void __launch_bounds__(32 * T, kTeamBlocksPerSM<T>) phase_team_kernel(const __grid_constant__ PhaseArgs a) {
+  extern __shared__ float dyn[];
+  __shared__ TeamShared<T> sh;
+  const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  int npairs = 0;
+  const int y = blockIdx.y * 4 + (lane >> 3);
+  update_team<kHalf, kTex, T>(a, sh, dyn, w, blockIdx.x * 16 + 2 * (lane & 7) + ((y + a.color) & 1), y, &npairs);
+  count_pairs(a, npairs);
+}
+template <bool kHalf, bool kTex, int T>
+__global__ void __launch_bounds__(32 * T, kTeamBlocksPerSM<T>) init_team_kernel(const __grid_constant__ PhaseArgs a) {
+  extern __shared__ float dyn[];
+  __shared__ TeamShared<T> sh;
+  const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  int npairs = 0;
+  init_team<kHalf, kTex, T>(a, sh, dyn, w, blockIdx.x * 8 + (lane & 7), blockIdx.y * 4 + (lane >> 3), &npairs);
+  count_pairs(a, npairs);
+}
 
 }  // namespace
 
@@ -90,9 +114,62 @@ void prefer_carveout(K kernel, int blocks, int smem, std::once_flag* once) {
   });
 }
 
+// Warps per 32 pixels for a launch over `groups` groups of 32 pixels: 16, 8 or 4
+// (a team), or 1 (one thread per pixel).  A team's fixed work (propagation,
+// window, view selection, barriers) is repeated or waited for by its warps, so
+// it pays while the GPU has room for it: 16 or 8 warps while all teams fit at
+// once with 16 warps per SM, 4 up to 0.8 of the warps that one thread per pixel
+// can keep resident (0.4 with fewer than four views, where the fixed work
+// weighs more).  Six sources, four iterations, 1 / 4 / 8 / 16 warps in us:
+// 64x48 750 / 328 / 233 / 229, 160x120 802 / 385 / 324 / 414, 320x240 1143 /
+// 1018 / 1078 / 1474, 400x300 1683 / 1563 / 1635 / 2299, 440x330 1748 / 1880 /
+// 1951 / 2794; with two sources 320x240 takes 462 / 501 / 611 / 972.
+int team_warps(int groups, int n_src) {
+  static int n_sm[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!n_sm[dev & 63]) cudaDeviceGetAttribute(&n_sm[dev & 63], cudaDevAttrMultiProcessorCount, dev);
+  const int warps = 16 * n_sm[dev & 63];
+  if (groups * 16 <= warps) return 16;
+  if (groups * 8 <= warps) return 8;
+  return groups * 10 <= warps * (n_src < 4 ? 4 : 8) ? 4 : 1;
+}
+// the team kernels' dynamic shared memory goes past the default limit with
+// many views; set once per device
+template <typename K>
+void allow_dynamic(K kernel, std::once_flag* once) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::call_once(once[dev & 63], [=] {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, team_floats(kMaxSrc) * (int)sizeof(float));
+  });
+}
+template <bool kHalf, bool kTex, int T>
+int launch_init_team(const PhaseArgs& a, cudaStream_t s) {
+  static std::once_flag once[64];
+  allow_dynamic(init_team_kernel<kHalf, kTex, T>, once);
+  const dim3 grid((a.W + 7) / 8, (a.H + 3) / 4);
+  init_team_kernel<kHalf, kTex, T><<<grid, 32 * T, kTeamPixels * a.N * sizeof(float), s>>>(a);
+  return (int)cudaGetLastError();
+}
+template <bool kHalf, bool kTex, int T>
+int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
+  static std::once_flag once[64];
+  allow_dynamic(phase_team_kernel<kHalf, kTex, T>, once);
+  const dim3 grid((a.W + 15) / 16, (a.H + 3) / 4);
+  phase_team_kernel<kHalf, kTex, T><<<grid, 32 * T, team_floats(a.N) * sizeof(float), s>>>(a);
+  return (int)cudaGetLastError();
+}
+
 template <bool kHalf, bool kTex>
 int launch_init_t(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
+  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N)) {
+    case 16: return launch_init_team<kHalf, kTex, 16>(a, s);
+    case 8: return launch_init_team<kHalf, kTex, 8>(a, s);
+    case 4: return launch_init_team<kHalf, kTex, 4>(a, s);
+    default: break;
+  }
   prefer_carveout(init_kernel<kHalf, kTex>, kPhaseBlocksPerSM, (int)sizeof(WinShared), once);
   dim3 grid((a.W + kTile - 1) / kTile, (a.H + 7) / 8);
   init_kernel<kHalf, kTex><<<grid, kThreads, 0, s>>>(a);
@@ -108,6 +185,14 @@ int launch_init(const PhaseArgs& a, cudaStream_t s) {
 template <bool kHalf, int kMode>
 int launch_phase_t(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
+  if constexpr (kMode == 0 || kMode == kTexture) {   // the ablations and the staged sweep: one thread per pixel
+    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N)) {
+      case 16: return launch_phase_team<kHalf, kMode == kTexture, 16>(a, s);
+      case 8: return launch_phase_team<kHalf, kMode == kTexture, 8>(a, s);
+      case 4: return launch_phase_team<kHalf, kMode == kTexture, 4>(a, s);
+      default: break;
+    }
+  }
   constexpr bool kStaged = (kMode & kStage) != 0;
   prefer_carveout(phase_kernel<kHalf, kMode>, kStaged ? kStagedBlocksPerSM : kPhaseBlocksPerSM,
                   (int)(sizeof(WinShared) + (kStaged ? sizeof(StageShared) : 0)), once);

@@ -623,8 +623,9 @@ __device__ __forceinline__ void joint_view_selection(const A& a, PixelArrays& sm
 }
 
 
-// mean of the k smallest of m[0..N), summed in ascending order (ties: lower
-// index) -- the heuristic view selection of Sec. 2
+// mean of the k smallest of m[0], m[kStep], ... (N of them), summed in
+// ascending order (ties: lower index) -- the heuristic view selection of Sec. 2
+template <int kStep = 1>
 __device__ __forceinline__ float kbest_mean(const float* m, int N, int k) {
   uint32_t used = 0;
   float acc = 0.f;
@@ -632,7 +633,7 @@ __device__ __forceinline__ float kbest_mean(const float* m, int N, int k) {
     int bj = -1;
     float bmv = 0.f;
     for (int j = 0; j < N; j++) {
-      const float mj = m[j];
+      const float mj = m[j * kStep];
       if (!(used >> j & 1u) && (bj < 0 || mj < bmv)) { bj = j; bmv = mj; }
     }
     used |= 1u << bj;
@@ -948,42 +949,34 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
 // depth uniform in [d_min, d_max], normal uniform on the sphere flipped to
 // face the camera, draws (pixel, 0, 0, 0); the initial cost is the mean of the
 // k smallest per-view costs, summed in ascending order (ties: lower view).
+template <class A>
+__device__ __forceinline__ float4 random_plane(const A& a, int x, int y, float3 ray) {
+  const uint4 r = philox4x32_10(make_uint4((uint32_t)(y * a.W + x), 0u, 0u, 0u), a.key0, a.key1);
+  const float3 n = face_camera(normal_from_uniforms(u01(r.y), u01(r.z)), ray);
+  return make_float4(n.x, n.y, n.z, a.dmin + (a.dmax - a.dmin) * u01(r.x));
+}
+template <class A>
+__device__ __forceinline__ void init_state(const A& a, int x, int y, float4 pl, float cost) {
+  const size_t pi = checked_index(a, state_index(x, y, a.W), state_size(a.W, a.H), kBadPixel);
+  a.plane[pi] = pl;
+  a.cost[pi] = cost;
+  a.sel[pi] = 0;
+  a.vbest[pi] = 255;
+  a.wmask[pi] = 0;
+  a.choice[pi] = 8;
+}
 template <bool kHalf, bool kTex, class A>
 __device__ __forceinline__ void init_pixel(const A& a, PixelArrays& sm, int x, int y, int* npairs, float4* win) {
   const int N = a.N;
-  const size_t pi = checked_index(a, state_index(x, y, a.W), state_size(a.W, a.H), kBadPixel);
-  const float fx = (float)x, fy = (float)y;
-  const float3 ray = ref_ray(a.Kinv, fx, fy);
-  const uint4 r = philox4x32_10(make_uint4((uint32_t)(y * a.W + x), 0u, 0u, 0u), a.key0, a.key1);
-  const float3 n = face_camera(normal_from_uniforms(u01(r.y), u01(r.z)), ray);
-  const float4 pl = make_float4(n.x, n.y, n.z, a.dmin + (a.dmax - a.dmin) * u01(r.x));
+  const float3 ray = ref_ray(a.Kinv, (float)x, (float)y);
+  const float4 pl = random_plane(a, x, y, ray);
   float4 c;
   const bool ok = plane_c(a.Kinv, pl, ray, &c);
   PixelWin rw;
   rw.q = win;
   load_ref_window<kHalf>(a, x, y, rw);
   for (int j = 0; j < N; j++) sm.wt(j) = ncc_cost<kHalf, kTex>(a.v[j], c, ok, ray, rw, npairs);
-  // mean of the k smallest per-view costs, summed in ascending order (ties:
-  // lower view index)
-  const int k = a.k < N ? a.k : N;
-  uint32_t used = 0;
-  float acc = 0.f;
-  for (int r2 = 0; r2 < k; r2++) {
-    int bj = -1;
-    float bmv = 0.f;
-    for (int j = 0; j < N; j++) {
-      const float mj = sm.wt(j);
-      if (!(used >> j & 1u) && (bj < 0 || mj < bmv)) { bj = j; bmv = mj; }
-    }
-    used |= 1u << bj;
-    acc += bmv;
-  }
-  a.plane[pi] = pl;
-  a.cost[pi] = acc / (float)k;
-  a.sel[pi] = 0;
-  a.vbest[pi] = 255;
-  a.wmask[pi] = 0;
-  a.choice[pi] = 8;
+  init_state(a, x, y, pl, kbest_mean(sm.w, N, a.k < N ? a.k : N));
 }
 
 }  // namespace upd

@@ -147,27 +147,46 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
 
-// Store one 32-byte sector per pixel (16 BF16 or 8 FP32 channels, as two
-// 16-byte halves lo, hi) for the pixels of lane pairs (2k, 2k + 1), which
-// are neighbours, so that each store instruction writes whole sectors: the
-// first writes the even pixel's sector (its lo from the even lane, its hi
-// from the odd one), the second the odd pixel's.  self / partner point at
-// this lane's and the pair partner's sector; st_self / st_partner say
-// whether those pixels are stored.  All 32 lanes call it together.
-__device__ __forceinline__ void store_sector_pair(uint4* self, uint4* partner, uint4 lo, uint4 hi, bool odd,
-                                                  bool st_self, bool st_partner) {
-  const uint4 send = odd ? lo : hi;    // the half the partner stores for this lane's pixel
-  uint4 recv;
-  recv.x = __shfl_xor_sync(0xffffffffu, send.x, 1);
-  recv.y = __shfl_xor_sync(0xffffffffu, send.y, 1);
-  recv.z = __shfl_xor_sync(0xffffffffu, send.z, 1);
-  recv.w = __shfl_xor_sync(0xffffffffu, send.w, 1);
-  uint4* const pa = odd ? partner + 1 : self;      // the even pixel's sector
-  uint4* const pb = odd ? self + 1 : partner;      // the odd pixel's sector
-  const uint4 va = odd ? recv : lo, vb = odd ? hi : recv;
-  const bool sa = odd ? st_partner : st_self, sb = odd ? st_self : st_partner;
-  if (sa) *pa = va;
-  if (sb) *pb = vb;
+// Lane pairs (2k, 2k + 1) hold neighbouring pixels, each lane its pixel's
+// 32-byte sector (16 BF16 channels) as two 16-byte halves lo, hi.  After the
+// exchange the even lane holds both pixels' lo, the odd lane both pixels' hi
+// (a of the even pixel, b of the odd one), so that storing a and then b at the
+// lane's half writes whole sectors with each instruction.  All 32 lanes call it.
+struct SectorPair {
+  uint4 a, b;
+};
+__device__ __forceinline__ uint4 shfl_xor1(uint4 v) {
+  return make_uint4(__shfl_xor_sync(0xffffffffu, v.x, 1), __shfl_xor_sync(0xffffffffu, v.y, 1),
+                    __shfl_xor_sync(0xffffffffu, v.z, 1), __shfl_xor_sync(0xffffffffu, v.w, 1));
+}
+__device__ __forceinline__ SectorPair pair_exchange(uint4 lo, uint4 hi, bool odd) {
+  const uint4 recv = shfl_xor1(odd ? lo : hi);
+  return odd ? SectorPair{recv, hi} : SectorPair{lo, recv};
+}
+// the programmatic dependent launch: the next kernel of the stream may start
+// its set-up once every block has called pdl_launch; pdl_wait returns when the
+// kernel before has finished and its writes are visible
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ float2 unpack_bf16(uint32_t v) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v));
+}
+// eight values as BF16 (16 bytes), and back
+__device__ __forceinline__ uint4 pack8(const float* f) {
+  return make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+}
+__device__ __forceinline__ void unpack8(uint4 v, float* f) {
+  const float2 a = unpack_bf16(v.x), b = unpack_bf16(v.y), c = unpack_bf16(v.z), d = unpack_bf16(v.w);
+  f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y; f[4] = c.x; f[5] = c.y; f[6] = d.x; f[7] = d.y;
+}
+__device__ __forceinline__ void store8(float* p, const float* f) {
+  reinterpret_cast<float4*>(p)[0] = make_float4(f[0], f[1], f[2], f[3]);
+  reinterpret_cast<float4*>(p)[1] = make_float4(f[4], f[5], f[6], f[7]);
 }
 
 // Forward / data-gradient kernel.  A tile is 128 consecutive pixels of one
@@ -196,12 +215,27 @@ constexpr int kConvMaxNb = 64;              // output channels per CTA
 __host__ __device__ constexpr int conv_threads(int nb) { return 32 * (4 * (nb / 16) + 2); }
 constexpr int kConvMaxThreads = 32 * (4 * (kConvMaxNb / 16) + 2);
 
+// What the epilogue does with a pixel's accumulator.  The encoder layers also
+// write the 2 x 2 mean the next level reads, the decoder layers the nearest
+// upsampling the next layer reads (instead of, or beside, their own output):
+// as passes of their own these took 70 of the forward's 225 us of kernels at
+// 800 x 528.
+enum ConvEpi {
+  kEpiPlain,    // y32
+  kEpiPool,     // y16, and up / down: its 2 x 2 mean (H / 2, W / 2)
+  kEpiUp,       // y16, and its nearest upsampling (2 H, 2 W)
+  kEpiSkip,     // r16 before the skip addition, y16 after
+  kEpiSkipUp    // r16 before the skip addition, the upsampling of the sum
+};
+__host__ __device__ constexpr bool epi_row_pairs(int epi) { return epi == kEpiPool; }   // tiles come in vertical pairs
+
 struct ConvTcArgs {
   const float* bias;          // Cout or null
-  const __nv_bfloat16* skip;  // (H, W, Cout) added after the ReLU, or null
-  __nv_bfloat16* y16;         // (H, W, Cout) BF16 output (after ReLU + skip), or null
-  __nv_bfloat16* r16;         // (H, W, Cout) ReLU output before the skip, or null
-  float* y32;                 // (H, W, Cout) FP32 output, or null
+  const __nv_bfloat16* skip;  // (H, W, Cout) added after the ReLU
+  __nv_bfloat16* y16;         // (H, W, Cout) BF16 output (after ReLU + skip)
+  __nv_bfloat16* r16;         // (H, W, Cout) ReLU output before the skip
+  __nv_bfloat16* res16;       // the 2 x 2 mean or the upsampling of the output
+  float* y32;                 // (H, W, Cout) FP32 output
   unsigned int* status;       // bit 0: a barrier wait gave up
   int H, W, Cin, Cout, relu;
   int Nb;                     // output channels per CTA (a multiple of 16 dividing Cout, at most kConvMaxNb)
@@ -242,11 +276,7 @@ __device__ __forceinline__ bool next_run(int& u, int hi, int H, TileRun& r) {
 // tx_main / tw_main: boxes of 64 channels x (kHalo pixels | Nb output
 // channels), 128-byte swizzle; tx_tail / tw_tail: the same for the tail
 // channels (unused when Cin is a multiple of 64)
-// kPairStores: the epilogue writes whole 32-byte sectors through lane pairs
-// (store_sector_pair); it pays where the stores bound the layer (the decoder
-// layers with a skip input and two BF16 outputs) and costs registers and
-// shuffles elsewhere
-template <bool kPairStores>
+template <int kEpi>
 __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tx_main,
                                                               const __grid_constant__ CUtensorMap tx_tail,
                                                               const __grid_constant__ CUtensorMap tw_main,
@@ -266,8 +296,10 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
   const int w_prod = 4 * (Nb / 16), w_mma = w_prod + 1;
   const int co0 = blockIdx.y * Nb;
   const int nseg = (a.W + kM - 1) / kM, ntiles = a.H * nseg;
-  const int lo = (int)((int64_t)ntiles * blockIdx.x / gridDim.x);
-  const int hi = (int)((int64_t)ntiles * (blockIdx.x + 1) / gridDim.x);
+  // with row pairs (H even) every range starts and ends at an even row
+  constexpr int kUnit = epi_row_pairs(kEpi) ? 2 : 1;
+  const int lo = kUnit * (int)((int64_t)(ntiles / kUnit) * blockIdx.x / gridDim.x);
+  const int hi = kUnit * (int)((int64_t)(ntiles / kUnit) * (blockIdx.x + 1) / gridDim.x);
   const uint32_t ncols = conv_acc_cols(Nb);
 
   if (warp == w_mma) {
@@ -297,11 +329,14 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
   if (warp == w_prod) {
     // producer: the weights once, then the slabs of every run in order
     if (lane == 0) {
+      // the weights are no output of the kernel before
       mbar_expect_tx(&wbar, 9u * (uint32_t)Nb * 2u * (uint32_t)a.Cin);
       for (int t = 0; t < 9; t++)
         for (int bk = 0; bk < nblk; bk++)
           tma_load_3d(wsm + (size_t)t * wtap_bytes + (size_t)bk * wblk, bk < nmain ? &tw_main : &tw_tail, 64 * bk, co0, t,
                       &wbar);
+      pdl_wait();
+      pdl_launch();
       RingPos q{0u, 0u};
       TileRun r;
       for (int u = lo; ok && next_run(u, hi, a.H, r);) {
@@ -381,8 +416,12 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
   } else {
     // epilogue: warp w drains TMEM lanes (pixels) 32 qw .. 32 qw + 31, qw =
     // w % 4, of output channels c0 .. c0 + 15, c0 = 16 (w / 4), of each tile
+    pdl_wait();
+    pdl_launch();
     const int qw = warp & 3, c0 = 16 * (warp >> 2);
+    constexpr bool kSkipIn = kEpi == kEpiSkip || kEpi == kEpiSkipUp;
     uint32_t tc = 0;
+    [[maybe_unused]] uint4 plo, phi;      // kEpiPool: the even row's output of this pixel
     TileRun r;
     for (int u = lo; ok && next_run(u, hi, a.H, r);) {
       for (int i = 0; i < r.len && ok; i++, tc++) {
@@ -391,8 +430,8 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
         const bool in = px < a.W;
         const size_t o = ((size_t)y * a.W + (in ? px : 0)) * a.Cout + co0 + c0;
         // this lane's skip values, fetched while the tile's MMAs run
-        uint4 sk0 = make_uint4(0, 0, 0, 0), sk1 = sk0;
-        if (a.skip && in) {
+        [[maybe_unused]] uint4 sk0, sk1;
+        if (kSkipIn) {
           sk0 = __ldg(reinterpret_cast<const uint4*>(a.skip + o));
           sk1 = __ldg(reinterpret_cast<const uint4*>(a.skip + o) + 1);
         }
@@ -406,68 +445,85 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[b]);
-        if (!kPairStores && !in) continue;
-        // with paired stores every lane goes on (the stores pair neighbouring
-        // lanes); lanes past the row's end compute on their TMEM rows and
-        // store only their partner's pixel
-        const bool odd = (lane & 1) != 0;
-        const bool in_partner = kPairStores ? __shfl_xor_sync(0xffffffffu, in ? 1 : 0, 1) != 0 : false;
-        const ptrdiff_t po = odd ? -(ptrdiff_t)a.Cout : (ptrdiff_t)a.Cout;   // the partner pixel's offset
-        // store offsets from the unclamped pixel (px - 1 <= W - 1 for the
-        // partner of a lane past the row's end)
-        const size_t os = ((size_t)y * a.W + px) * a.Cout + co0 + c0;
         float f[16];
 #pragma unroll
         for (int e = 0; e < 16; e++) {
           const float val = __uint_as_float(v[e]) + bias_s[c0 + e];
           f[e] = a.relu ? fmaxf(val, 0.f) : val;
         }
-        __align__(16) __nv_bfloat16 hb[16];
-        if (a.r16) {
-#pragma unroll
-          for (int e = 0; e < 16; e++) hb[e] = __float2bfloat16(f[e]);
-          if constexpr (kPairStores) {
-            store_sector_pair(reinterpret_cast<uint4*>(a.r16 + os), reinterpret_cast<uint4*>(a.r16 + os + po),
-                              reinterpret_cast<const uint4*>(hb)[0], reinterpret_cast<const uint4*>(hb)[1], odd, in,
-                              in_partner);
-          } else {
-            reinterpret_cast<uint4*>(a.r16 + o)[0] = reinterpret_cast<const uint4*>(hb)[0];
-            reinterpret_cast<uint4*>(a.r16 + o)[1] = reinterpret_cast<const uint4*>(hb)[1];
+        if constexpr (kEpi == kEpiPlain) {
+          if (in) {
+            store8(a.y32 + o, f);
+            store8(a.y32 + o + 8, f + 8);
           }
+          continue;
         }
-        if (a.skip) {
-          __align__(16) __nv_bfloat16 skb[16];
-          reinterpret_cast<uint4*>(skb)[0] = sk0;
-          reinterpret_cast<uint4*>(skb)[1] = sk1;
-#pragma unroll
-          for (int e = 0; e < 16; e++) f[e] = __bfloat162float(__float2bfloat16(f[e])) + __bfloat162float(skb[e]);
-        }
-        if (a.y16) {
-#pragma unroll
-          for (int e = 0; e < 16; e++) hb[e] = __float2bfloat16(f[e]);
-          if constexpr (kPairStores) {
-            store_sector_pair(reinterpret_cast<uint4*>(a.y16 + os), reinterpret_cast<uint4*>(a.y16 + os + po),
-                              reinterpret_cast<const uint4*>(hb)[0], reinterpret_cast<const uint4*>(hb)[1], odd, in,
-                              in_partner);
-          } else {
-            reinterpret_cast<uint4*>(a.y16 + o)[0] = reinterpret_cast<const uint4*>(hb)[0];
-            reinterpret_cast<uint4*>(a.y16 + o)[1] = reinterpret_cast<const uint4*>(hb)[1];
+        // Lanes past the row's end compute on their TMEM rows and take part in
+        // the exchanges; they store only their partner's pixel.
+        const bool odd = (lane & 1) != 0;
+        uint4 h0 = pack8(f), h1 = pack8(f + 8);
+        if constexpr (kEpi == kEpiPool) {
+          // W and H are even: both pixels and both rows of a pair are inside.
+          // The even lane averages channels 0-7, the odd lane 8-15.
+          if (in) {
+            reinterpret_cast<uint4*>(a.y16 + o)[0] = h0;
+            reinterpret_cast<uint4*>(a.y16 + o)[1] = h1;
           }
-        }
-        if (a.y32 && !kPairStores) {
-          float4* q4 = reinterpret_cast<float4*>(a.y32 + o);
+          if (y & 1) {
+            const uint4 r0 = shfl_xor1(odd ? plo : phi), r1 = shfl_xor1(odd ? h0 : h1);
+            float x00[8], x01[8], x10[8], x11[8], m[8];
+            unpack8(odd ? r0 : plo, x00);
+            unpack8(odd ? phi : r0, x01);
+            unpack8(odd ? r1 : h0, x10);
+            unpack8(odd ? h1 : r1, x11);
 #pragma unroll
-          for (int e = 0; e < 4; e++) q4[e] = make_float4(f[4 * e], f[4 * e + 1], f[4 * e + 2], f[4 * e + 3]);
-        }
-        if (a.y32 && kPairStores) {   // two sectors: channels 0-7 and 8-15
+            for (int e = 0; e < 8; e++) m[e] = 0.25f * (((x00[e] + x01[e]) + x10[e]) + x11[e]);
+            if (in)
+              *reinterpret_cast<uint4*>(a.res16 + ((size_t)(y >> 1) * (a.W >> 1) + (px >> 1)) * a.Cout + co0 + c0 +
+                                        (odd ? 8 : 0)) = pack8(m);
+          } else {
+            plo = h0;
+            phi = h1;
+          }
+        } else {
+          // the lane's half (lo: even lanes, hi: odd lanes) of the sectors of the
+          // pair's two pixels
+          const bool in_partner = __shfl_xor_sync(0xffffffffu, in ? 1 : 0, 1) != 0;
+          const bool in_a = odd ? in_partner : in, in_b = odd ? in : in_partner;
+          const int xa = px & ~1, half = odd ? 8 : 0;
+          const size_t oa = ((size_t)y * a.W + xa) * a.Cout + co0 + c0 + half;
+          SectorPair q = pair_exchange(h0, h1, odd);
+          if constexpr (kSkipIn) {
+            if (in_a) *reinterpret_cast<uint4*>(a.r16 + oa) = q.a;
+            if (in_b) *reinterpret_cast<uint4*>(a.r16 + oa + a.Cout) = q.b;
+            float s[16];
+            unpack8(h0, f);
+            unpack8(h1, f + 8);
+            unpack8(sk0, s);
+            unpack8(sk1, s + 8);
 #pragma unroll
-          for (int h = 0; h < 2; h++) {
-            const uint4 lo = make_uint4(__float_as_uint(f[8 * h]), __float_as_uint(f[8 * h + 1]),
-                                        __float_as_uint(f[8 * h + 2]), __float_as_uint(f[8 * h + 3]));
-            const uint4 hi = make_uint4(__float_as_uint(f[8 * h + 4]), __float_as_uint(f[8 * h + 5]),
-                                        __float_as_uint(f[8 * h + 6]), __float_as_uint(f[8 * h + 7]));
-            store_sector_pair(reinterpret_cast<uint4*>(a.y32 + os + 8 * h), reinterpret_cast<uint4*>(a.y32 + os + po + 8 * h),
-                              lo, hi, odd, in, in_partner);
+            for (int e = 0; e < 16; e++) f[e] = f[e] + s[e];
+            h0 = pack8(f);
+            h1 = pack8(f + 8);
+            q = pair_exchange(h0, h1, odd);
+          }
+          if constexpr (kEpi == kEpiUp || kEpi == kEpiSkip) {
+            if (in_a) *reinterpret_cast<uint4*>(a.y16 + oa) = q.a;
+            if (in_b) *reinterpret_cast<uint4*>(a.y16 + oa + a.Cout) = q.b;
+          }
+          if constexpr (kEpi == kEpiUp || kEpi == kEpiSkipUp) {
+#pragma unroll
+            for (int dy = 0; dy < 2; dy++) {
+              __nv_bfloat16* d = a.res16 + ((size_t)(2 * y + dy) * (2 * a.W) + 2 * xa) * a.Cout + co0 + c0 + half;
+              if (in_a) {
+                *reinterpret_cast<uint4*>(d) = q.a;
+                *reinterpret_cast<uint4*>(d + a.Cout) = q.a;
+              }
+              if (in_b) {
+                *reinterpret_cast<uint4*>(d + 2 * a.Cout) = q.b;
+                *reinterpret_cast<uint4*>(d + 3 * a.Cout) = q.b;
+              }
+            }
           }
         }
       }

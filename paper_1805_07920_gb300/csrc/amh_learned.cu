@@ -122,30 +122,12 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 __device__ __forceinline__ float4 scale4(float s, float4 a) { return make_float4(s * a.x, s * a.y, s * a.z, s * a.w); }
 
-__global__ void pool2_kernel(const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ y, int H, int W, int C) {
-  const int Ho = H / 2, Wo = W / 2;
-  const size_t n = (size_t)Ho * Wo * C / 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(4 * i % C), p = (int)(4 * i / C), oy = p / Wo, ox = p % Wo;
-    const size_t b = ((size_t)(2 * oy) * W + 2 * ox) * C + c;
-    const float4 s = add4(add4(add4(ld4(x + b), ld4(x + b + C)), ld4(x + b + (size_t)W * C)), ld4(x + b + (size_t)W * C + C));
-    st4(y + 4 * i, scale4(0.25f, s));
-  }
-}
 __global__ void pool2_bwd_add_kernel(const float* __restrict__ d, float* __restrict__ dx, int H, int W, int C) {   // dx += pool'^T d
   const size_t n = (size_t)H * W * C / 4;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const int c = (int)(4 * i % C), p = (int)(4 * i / C), yy = p / W, xx = p % W;
     float4* o = reinterpret_cast<float4*>(dx) + i;
     *o = add4(*o, scale4(0.25f, *reinterpret_cast<const float4*>(d + ((size_t)(yy / 2) * (W / 2) + xx / 2) * C + c)));
-  }
-}
-__global__ void up2_kernel(const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ y, int Ho, int Wo, int C) {  // (Ho, Wo) output
-  const size_t n = (size_t)Ho * Wo * C / 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(4 * i % C), p = (int)(4 * i / C), yy = p / Wo, xx = p % Wo;
-    *reinterpret_cast<bf16x4*>(y + 4 * i) =
-        *reinterpret_cast<const bf16x4*>(x + ((size_t)(yy / 2) * (Wo / 2) + xx / 2) * C + c);
   }
 }
 __global__ void up2_bwd_kernel(const float* __restrict__ d, float* __restrict__ dx, int H, int W, int C) {   // (H, W) = input size
@@ -175,6 +157,14 @@ __global__ void relu_mask_kernel(const float* __restrict__ g, const __nv_bfloat1
 __global__ void bf16_to_f32_kernel(const __nv_bfloat16* g, float* o, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     o[i] = __bfloat162float(g[i]);
+}
+// out (H, W, C) FP32: pixels (2 x, 2 y) of the BF16 tensor x (2 H, 2 W, C)
+__global__ void subsample_kernel(const __nv_bfloat16* x, float* o, int H, int W, int C) {
+  const size_t n = (size_t)H * W * C;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t p = i / C;
+    o[i] = __bfloat162float(x[((2 * (p / W)) * (2 * W) + 2 * (p % W)) * C + i % C]);
+  }
 }
 __global__ void to_bf16_kernel(const float* g, __nv_bfloat16* o, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -324,6 +314,16 @@ using namespace amh;
 // ===========================================================================
 // host side
 // ===========================================================================
+// One convolution of the network, laid out once: its tensor maps, arguments
+// and launch shape depend only on the network's own buffers.
+struct ConvOp {
+  CUtensorMap mx[2], mw[2];
+  tc::ConvTcArgs a;
+  int epi;
+  dim3 grid;
+  int threads;
+  size_t smem;
+};
 struct amh_net {
   int w2 = 0, h2 = 0;                     // network input size (half resolution)
   cudaStream_t stream = nullptr;
@@ -338,8 +338,8 @@ struct amh_net {
   int step = 0;
   // activations (BF16) and gradient buffers (FP32)
   __nv_bfloat16 *x0 = nullptr, *e1 = nullptr, *in_e2 = nullptr, *e2 = nullptr, *in_e3 = nullptr, *e3 = nullptr,
-                *in_e4 = nullptr, *e4 = nullptr, *in_d3 = nullptr, *r3 = nullptr, *d3 = nullptr, *in_d2 = nullptr,
-                *r2 = nullptr, *d2 = nullptr, *in_d1 = nullptr, *r1 = nullptr, *d1 = nullptr, *g16 = nullptr;
+                *in_e4 = nullptr, *e4 = nullptr, *in_d3 = nullptr, *r3 = nullptr, *in_d2 = nullptr,
+                *r2 = nullptr, *in_d1 = nullptr, *r1 = nullptr, *d1 = nullptr, *g16 = nullptr;
   float* out = nullptr;
   float* target = nullptr;
   uint8_t* mask = nullptr;
@@ -349,6 +349,7 @@ struct amh_net {
   // gA / gB scratch, gE1..gE3 gradients arriving at e1..e3 through the skips
   float* dy[kLayers] = {};
   float *gA = nullptr, *gB = nullptr, *gE1 = nullptr, *gE2 = nullptr, *gE3 = nullptr;
+  ConvOp fwd[kLayers], dgr[kLayers];      // forward; data gradients (layer 0 has none)
   float* loss = nullptr;
   unsigned int* status = nullptr;         // bit 0: a convolution's barrier wait gave up
   size_t maxel = 0;
@@ -418,69 +419,128 @@ CUtensorMapSwizzle block_swizzle(int nch) {
   return nch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : nch == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
 }
 
-// 3x3 convolution on the tensor cores (amh_conv_tc.cuh): x (H, W, Cin), w (9,
-// Cout, Cin), Cin and Cout multiples of 16, Cout at most 128
-int conv(amh_net* n, const __nv_bfloat16* x, const __nv_bfloat16* w, const float* bias, const __nv_bfloat16* skip,
-         __nv_bfloat16* y16, __nv_bfloat16* r16, float* y32, int H, int W, int Cin, int Cout, int relu) {
+// the convolution kernels, by epilogue
+const void* conv_kernel(int epi) {
+  switch (epi) {
+    case tc::kEpiPool: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiPool>);
+    case tc::kEpiUp: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiUp>);
+    case tc::kEpiSkip: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiSkip>);
+    case tc::kEpiSkipUp: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiSkipUp>);
+    default: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiPlain>);
+  }
+}
+// Launch of a convolution.  overlap: its set-up (barriers, tensor memory,
+// weights) may start while the kernel before it on the stream is still running;
+// the kernel itself waits for that one before it reads or writes anything else.
+// The weights are read during set-up, so they must be complete one ordinary
+// launch earlier: the first convolution after they may have changed does not
+// overlap.
+cudaError_t launch_conv(const void* kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, bool overlap, void** args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
+// Lay out a 3x3 convolution on the tensor cores (amh_conv_tc.cuh): x (H, W,
+// Cin), w (9, Cout, Cin), Cin and Cout multiples of 16, Cout at most 128; a
+// holds the other tensors of the epilogue.
+int plan_conv(amh_net* n, ConvOp& op, const __nv_bfloat16* x, const __nv_bfloat16* w, int H, int W, int Cin, int Cout,
+              int epi, tc::ConvTcArgs a) {
   if (Cin % 16 || Cin > 128 || Cin % 64 == 48 || Cout % 16 || Cout > tc::kMaxCout)
     return nfail(n, AMH_EINVAL, "conv: channel counts");
   const tc::ConvPlan p = tc::conv_plan(Cin, Cout);
   // one map per kind of channel block (64 channels; the 16 or 32 of the
   // tail); a kind the layer lacks gets a copy of the other
-  CUtensorMap mx[2], mw[2];
   const int tail = Cin % 64;
   bool ok = true;
   if (Cin >= 64)
-    ok = bf16_map(&mx[0], x, Cin, W, H, 64, tc::kHalo, 1, 0, block_swizzle(64)) &&
-         bf16_map(&mw[0], w, Cin, Cout, 9, 64, p.Nb, 1, 0, block_swizzle(64));
+    ok = bf16_map(&op.mx[0], x, Cin, W, H, 64, tc::kHalo, 1, 0, block_swizzle(64)) &&
+         bf16_map(&op.mw[0], w, Cin, Cout, 9, 64, p.Nb, 1, 0, block_swizzle(64));
   if (ok && tail)
-    ok = bf16_map(&mx[1], x, Cin, W, H, tail, tc::kHalo, 1, 0, block_swizzle(tail)) &&
-         bf16_map(&mw[1], w, Cin, Cout, 9, tail, p.Nb, 1, 0, block_swizzle(tail));
+    ok = bf16_map(&op.mx[1], x, Cin, W, H, tail, tc::kHalo, 1, 0, block_swizzle(tail)) &&
+         bf16_map(&op.mw[1], w, Cin, Cout, 9, tail, p.Nb, 1, 0, block_swizzle(tail));
   if (!ok) return nfail(n, AMH_ECUDA, "conv: tensor map encoding failed");
-  if (Cin < 64) mx[0] = mx[1], mw[0] = mw[1];
-  if (!tail) mx[1] = mx[0], mw[1] = mw[0];
-  const tc::ConvTcArgs a{bias, skip, y16, r16, y32, n->status, H, W, Cin, Cout, relu, p.Nb, p.S};
-  // persistent grid: per channel block, as many CTAs as fit on the SMs at
-  // once (every CTA holds its tensor memory until it exits), at most one per
-  // tile
-  static int n_sm[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (!n_sm[dev & 63]) cudaDeviceGetAttribute(&n_sm[dev & 63], cudaDevAttrMultiProcessorCount, dev);
-  // the decoder layers (skip input, two BF16 outputs) write their outputs
-  // in whole sectors through lane pairs (tc::store_sector_pair)
-  const int pair = skip ? 1 : 0;
-  static std::once_flag once[64];
-  static cudaError_t attr_err[64] = {};
-  static int regs[64][2] = {};
-  std::call_once(once[dev & 63], [dev] {
-    cudaError_t e = cudaSuccess;
-    cudaFuncAttributes fa;
-    const void* kerns[2] = {reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<false>),
-                            reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<true>)};
-    for (int k = 0; k < 2 && e == cudaSuccess; k++) {
-      e = cudaFuncSetAttribute(kerns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kConvSmemCap);
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kerns[k]);
-      if (e == cudaSuccess) regs[dev & 63][k] = fa.numRegs;
-    }
-    attr_err[dev & 63] = e;
-  });
-  if (attr_err[dev & 63] != cudaSuccess)
-    return nfail(n, AMH_ECUDA, "conv: shared-memory attribute: %s", cudaGetErrorString(attr_err[dev & 63]));
+  if (Cin < 64) op.mx[0] = op.mx[1], op.mw[0] = op.mw[1];
+  if (!tail) op.mx[1] = op.mx[0], op.mw[1] = op.mw[0];
+  a.status = n->status;
+  a.H = H;
+  a.W = W;
+  a.Cin = Cin;
+  a.Cout = Cout;
+  a.Nb = p.Nb;
+  a.S = p.S;
+  op.a = a;
+  op.epi = epi;
+  op.threads = tc::conv_threads(p.Nb);
+  op.smem = p.smem;
   if (p.smem > tc::kConvSmemCap) return nfail(n, AMH_EINVAL, "conv: shared memory plan too large");
-  // CTAs resident per SM: the plan's, and what the register file holds
-  const int threads = tc::conv_threads(p.Nb);
-  const int by_regs = 65536 / (((regs[dev & 63][pair] + 7) & ~7) * threads);
+  cudaFuncAttributes fa;
+  int dev = 0, n_sm = 0;
+  cudaError_t e = cudaFuncSetAttribute(conv_kernel(epi), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kConvSmemCap);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, conv_kernel(epi));
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "conv: kernel attributes: %s", cudaGetErrorString(e));
+  // persistent grid: per channel block, as many CTAs as fit on the SMs at
+  // once (every CTA holds its tensor memory until it exits), by the plan and by
+  // the register file; at most one per tile
+  const int by_regs = 65536 / (((fa.numRegs + 7) & ~7) * op.threads);
   const int cps = std::max(1, std::min(p.ctas_per_sm, by_regs));
   const int nblk = Cout / p.Nb, ntiles = H * ((W + tc::kM - 1) / tc::kM);
-  const int gx = std::max(1, std::min(ntiles, n_sm[dev & 63] * cps / nblk));
-  if (pair)
-    tc::conv3x3_tc_kernel<true><<<dim3(gx, nblk), threads, p.smem, n->stream>>>(mx[0], mx[1], mw[0], mw[1], a);
-  else
-    tc::conv3x3_tc_kernel<false><<<dim3(gx, nblk), threads, p.smem, n->stream>>>(mx[0], mx[1], mw[0], mw[1], a);
-  cudaError_t e = cudaGetLastError();
+  op.grid = dim3(std::max(1, std::min(ntiles, n_sm * cps / nblk)), nblk);
+  return AMH_OK;
+}
+int conv(amh_net* n, ConvOp& op, bool overlap) {
+  void* args[] = {&op.mx[0], &op.mx[1], &op.mw[0], &op.mw[1], &op.a};
+  const cudaError_t e = launch_conv(conv_kernel(op.epi), op.grid, op.threads, op.smem, n->stream, overlap, args);
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "conv launch: %s", cudaGetErrorString(e));
   return AMH_OK;
+}
+// every convolution of the forward and backward pass
+int plan_network(amh_net* n) {
+  const int W0 = n->w2, H0 = n->h2, W1 = W0 / 2, H1 = H0 / 2, W2 = W1 / 2, H2 = H1 / 2, W3 = W2 / 2, H3 = H2 / 2;
+  struct F {
+    const __nv_bfloat16* x;
+    int H, W, epi;
+    const __nv_bfloat16* skip;
+    __nv_bfloat16 *y16, *r16, *res16;
+    float* y32;
+  };
+  const F f[kLayers] = {{n->x0, H0, W0, tc::kEpiPool, nullptr, n->e1, nullptr, n->in_e2, nullptr},
+                        {n->in_e2, H1, W1, tc::kEpiPool, nullptr, n->e2, nullptr, n->in_e3, nullptr},
+                        {n->in_e3, H2, W2, tc::kEpiPool, nullptr, n->e3, nullptr, n->in_e4, nullptr},
+                        {n->in_e4, H3, W3, tc::kEpiUp, nullptr, n->e4, nullptr, n->in_d3, nullptr},
+                        {n->in_d3, H2, W2, tc::kEpiSkipUp, n->e3, nullptr, n->r3, n->in_d2, nullptr},
+                        {n->in_d2, H1, W1, tc::kEpiSkipUp, n->e2, nullptr, n->r2, n->in_d1, nullptr},
+                        {n->in_d1, H0, W0, tc::kEpiSkip, n->e1, n->d1, n->r1, nullptr, nullptr},
+                        {n->d1, H0, W0, tc::kEpiPlain, nullptr, nullptr, nullptr, nullptr, n->out}};
+  int rc = AMH_OK;
+  for (int L = 0; L < kLayers && !rc; L++) {
+    tc::ConvTcArgs a{};
+    a.bias = n->bm[L];
+    a.skip = f[L].skip;
+    a.y16 = f[L].y16;
+    a.r16 = f[L].r16;
+    a.res16 = f[L].res16;
+    a.y32 = f[L].y32;
+    a.relu = kNet[L].relu;
+    rc = plan_conv(n, n->fwd[L], f[L].x, n->w16[L], f[L].H, f[L].W, kNet[L].cin, kNet[L].cout, f[L].epi, a);
+  }
+  // data gradients: dx (FP32, H x W x Cin, in gA) from dy (BF16 copy in g16)
+  for (int L = 1; L < kLayers && !rc; L++) {
+    tc::ConvTcArgs a{};
+    a.y32 = n->gA;
+    rc = plan_conv(n, n->dgr[L], n->g16, n->wd16[L], f[L].H, f[L].W, kNet[L].cout, kNet[L].cin, tc::kEpiPlain, a);
+  }
+  return rc;
 }
 // weight gradient of layer L from its input x and its output gradient (FP32
 // dy for the bias, its BF16 copy dy16 for the weights): the tensor-core
@@ -522,10 +582,6 @@ int wgrad(amh_net* n, int L, const __nv_bfloat16* x, const float* dy, const __nv
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "wgrad launch: %s", cudaGetErrorString(e));
   return AMH_OK;
-}
-// data gradient of layer L: dx (FP32, H x W x Cin) from dy (BF16 copy in g16)
-int dgrad(amh_net* n, int L, const __nv_bfloat16* dy16, float* dx, int H, int W) {
-  return conv(n, dy16, n->wd16[L], nullptr, nullptr, nullptr, nullptr, dx, H, W, kNet[L].cout, kNet[L].cin, 0);
 }
 }  // namespace
 
@@ -579,7 +635,7 @@ AMH_API int amh_net_create(amh_net** out, int32_t width2, int32_t height2, uint6
   const size_t P0 = (size_t)width2 * height2, P1 = P0 / 4, P2 = P0 / 16, P3 = P0 / 64;
   NA(n->x0, P0 * 16); NA(n->e1, P0 * 32); NA(n->in_e2, P1 * 32); NA(n->e2, P1 * 64); NA(n->in_e3, P2 * 64);
   NA(n->e3, P2 * 96); NA(n->in_e4, P3 * 96); NA(n->e4, P3 * 128); NA(n->in_d3, P2 * 128); NA(n->r3, P2 * 96);
-  NA(n->d3, P2 * 96); NA(n->in_d2, P1 * 96); NA(n->r2, P1 * 64); NA(n->d2, P1 * 64); NA(n->in_d1, P0 * 64);
+  NA(n->in_d2, P1 * 96); NA(n->r2, P1 * 64); NA(n->in_d1, P0 * 64);
   NA(n->r1, P0 * 32); NA(n->d1, P0 * 32);
   n->maxel = P0 * 64;
   NA(n->g16, n->maxel); NA(n->gA, n->maxel); NA(n->gB, n->maxel);
@@ -590,6 +646,7 @@ AMH_API int amh_net_create(amh_net** out, int32_t width2, int32_t height2, uint6
   NA(n->gE1, P0 * 32); NA(n->gE2, P1 * 64); NA(n->gE3, P2 * 96);
   NA(n->out, P0 * 16); NA(n->target, P0 * 4); NA(n->mask, P0); NA(n->pin, P0); NA(n->prop, P0); NA(n->loss, 1);
 #undef NA
+  if (const int rc = plan_network(n)) return bail(rc);
   for (int L = 0; L < kLayers; L++) {
     const size_t nw = (size_t)9 * kNet[L].cin * kNet[L].cout;
     to_bf16_kernel<<<blocks_for(nw), 256, 0, n->stream>>>(n->wm[L], n->w16[L], nw);
@@ -699,26 +756,13 @@ AMH_API int amh_net_set_targets(amh_net* n, const float* target_host, const uint
 
 AMH_API int amh_net_forward(amh_net* n, float* out_host) {
   if (!n) return AMH_EINVAL;
-  const int W0 = n->w2, H0 = n->h2, W1 = W0 / 2, H1 = H0 / 2, W2 = W1 / 2, H2 = H1 / 2, W3 = W2 / 2, H3 = H2 / 2;
   const cudaStream_t s = n->stream;
-  int rc = conv(n, n->x0, n->w16[0], n->bm[0], nullptr, n->e1, nullptr, nullptr, H0, W0, 16, 32, 1);
-  pool2_kernel<<<blocks_for((size_t)H1 * W1 * 32), 256, 0, s>>>(n->e1, n->in_e2, H0, W0, 32);
-  if (!rc) rc = conv(n, n->in_e2, n->w16[1], n->bm[1], nullptr, n->e2, nullptr, nullptr, H1, W1, 32, 64, 1);
-  pool2_kernel<<<blocks_for((size_t)H2 * W2 * 64), 256, 0, s>>>(n->e2, n->in_e3, H1, W1, 64);
-  if (!rc) rc = conv(n, n->in_e3, n->w16[2], n->bm[2], nullptr, n->e3, nullptr, nullptr, H2, W2, 64, 96, 1);
-  pool2_kernel<<<blocks_for((size_t)H3 * W3 * 96), 256, 0, s>>>(n->e3, n->in_e4, H2, W2, 96);
-  if (!rc) rc = conv(n, n->in_e4, n->w16[3], n->bm[3], nullptr, n->e4, nullptr, nullptr, H3, W3, 96, 128, 1);
-  up2_kernel<<<blocks_for((size_t)H2 * W2 * 128), 256, 0, s>>>(n->e4, n->in_d3, H2, W2, 128);
-  if (!rc) rc = conv(n, n->in_d3, n->w16[4], n->bm[4], n->e3, n->d3, n->r3, nullptr, H2, W2, 128, 96, 1);
-  up2_kernel<<<blocks_for((size_t)H1 * W1 * 96), 256, 0, s>>>(n->d3, n->in_d2, H1, W1, 96);
-  if (!rc) rc = conv(n, n->in_d2, n->w16[5], n->bm[5], n->e2, n->d2, n->r2, nullptr, H1, W1, 96, 64, 1);
-  up2_kernel<<<blocks_for((size_t)H0 * W0 * 64), 256, 0, s>>>(n->d2, n->in_d1, H0, W0, 64);
-  if (!rc) rc = conv(n, n->in_d1, n->w16[6], n->bm[6], n->e1, n->d1, n->r1, nullptr, H0, W0, 64, 32, 1);
-  if (!rc) rc = conv(n, n->d1, n->w16[7], n->bm[7], nullptr, nullptr, nullptr, n->out, H0, W0, 32, 16, 0);
+  int rc = AMH_OK;
+  for (int L = 0; L < kLayers && !rc; L++) rc = conv(n, n->fwd[L], L > 0);
   if (rc) return rc;
   NTRY(n, cudaGetLastError());
   if (out_host) {
-    NTRY(n, cudaMemcpyAsync(out_host, n->out, (size_t)H0 * W0 * 16 * 4, cudaMemcpyDeviceToHost, s));
+    NTRY(n, cudaMemcpyAsync(out_host, n->out, (size_t)n->w2 * n->h2 * 16 * 4, cudaMemcpyDeviceToHost, s));
     NTRY(n, cudaStreamSynchronize(s));
   }
   return AMH_OK;
@@ -747,34 +791,34 @@ AMH_API int amh_net_backward(amh_net* n, float* loss_out) {
   // out = conv(d1)
   to_bf16_kernel<<<blocks_for(P0 * 16), 256, 0, s>>>(dy[7], n->g16, P0 * 16);
   int rc = wgrad(n, 7, n->d1, dy[7], n->g16, H0, W0);
-  if (!rc) rc = dgrad(n, 7, n->g16, n->gA, H0, W0);                  // gA = d d1 (P0 x 32)
+  if (!rc) rc = conv(n, n->dgr[7], false);                  // gA = d d1 (P0 x 32)
   // d1 = relu(conv(in_d1)) + e1
   NTRY(n, cudaMemcpyAsync(n->gE1, n->gA, P0 * 32 * 4, cudaMemcpyDeviceToDevice, s));
   relu_mask_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gA, n->r1, dy[6], n->g16, P0 * 32);
   if (!rc) rc = wgrad(n, 6, n->in_d1, dy[6], n->g16, H0, W0);
-  if (!rc) rc = dgrad(n, 6, n->g16, n->gA, H0, W0);                  // d in_d1 (P0 x 64)
+  if (!rc) rc = conv(n, n->dgr[6], false);                  // d in_d1 (P0 x 64)
   up2_bwd_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gA, n->gE2, H1, W1, 64);  // d d2 (P1 x 64)
   relu_mask_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gE2, n->r2, dy[5], n->g16, P1 * 64);
   if (!rc) rc = wgrad(n, 5, n->in_d2, dy[5], n->g16, H1, W1);
-  if (!rc) rc = dgrad(n, 5, n->g16, n->gA, H1, W1);                  // d in_d2 (P1 x 96)
+  if (!rc) rc = conv(n, n->dgr[5], false);                  // d in_d2 (P1 x 96)
   up2_bwd_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gA, n->gE3, H2, W2, 96);  // d d3 (P2 x 96)
   relu_mask_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gE3, n->r3, dy[4], n->g16, P2 * 96);
   if (!rc) rc = wgrad(n, 4, n->in_d3, dy[4], n->g16, H2, W2);
-  if (!rc) rc = dgrad(n, 4, n->g16, n->gA, H2, W2);                  // d in_d3 (P2 x 128)
+  if (!rc) rc = conv(n, n->dgr[4], false);                  // d in_d3 (P2 x 128)
   up2_bwd_kernel<<<blocks_for(P3 * 128), 256, 0, s>>>(n->gA, n->gB, H3, W3, 128); // d e4 (P3 x 128)
   // e4 = relu(conv(in_e4))
   relu_mask_kernel<<<blocks_for(P3 * 128), 256, 0, s>>>(n->gB, n->e4, dy[3], n->g16, P3 * 128);
   if (!rc) rc = wgrad(n, 3, n->in_e4, dy[3], n->g16, H3, W3);
-  if (!rc) rc = dgrad(n, 3, n->g16, n->gA, H3, W3);                  // d in_e4 (P3 x 96)
+  if (!rc) rc = conv(n, n->dgr[3], false);                  // d in_e4 (P3 x 96)
   pool2_bwd_add_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gA, n->gE3, H2, W2, 96);
   // e3 = relu(conv(in_e3)), read by d3 (skip) and by the pooling
   relu_mask_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gE3, n->e3, dy[2], n->g16, P2 * 96);
   if (!rc) rc = wgrad(n, 2, n->in_e3, dy[2], n->g16, H2, W2);
-  if (!rc) rc = dgrad(n, 2, n->g16, n->gA, H2, W2);                  // d in_e3 (P2 x 64)
+  if (!rc) rc = conv(n, n->dgr[2], false);                  // d in_e3 (P2 x 64)
   pool2_bwd_add_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gA, n->gE2, H1, W1, 64);
   relu_mask_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gE2, n->e2, dy[1], n->g16, P1 * 64);
   if (!rc) rc = wgrad(n, 1, n->in_e2, dy[1], n->g16, H1, W1);
-  if (!rc) rc = dgrad(n, 1, n->g16, n->gA, H1, W1);                  // d in_e2 (P1 x 32)
+  if (!rc) rc = conv(n, n->dgr[1], false);                  // d in_e2 (P1 x 32)
   pool2_bwd_add_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gA, n->gE1, H0, W0, 32);
   relu_mask_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gE1, n->e1, dy[0], n->g16, P0 * 32);
   if (!rc) rc = wgrad(n, 0, n->x0, dy[0], n->g16, H0, W0);
@@ -830,8 +874,8 @@ AMH_API int amh_net_read(amh_net* n, int32_t which, float* out, int64_t* count) 
   const B act[] = {{n->x0, nullptr, P0 * 16},   {n->e1, nullptr, P0 * 32},    {n->in_e2, nullptr, P1 * 32},
                    {n->e2, nullptr, P1 * 64},   {n->in_e3, nullptr, P2 * 64}, {n->e3, nullptr, P2 * 96},
                    {n->in_e4, nullptr, P3 * 96}, {n->e4, nullptr, P3 * 128},  {n->in_d3, nullptr, P2 * 128},
-                   {n->r3, nullptr, P2 * 96},   {n->d3, nullptr, P2 * 96},    {n->in_d2, nullptr, P1 * 96},
-                   {n->r2, nullptr, P1 * 64},   {n->d2, nullptr, P1 * 64},    {n->in_d1, nullptr, P0 * 64},
+                   {n->r3, nullptr, P2 * 96},   {n->in_d2, nullptr, P2 * 96},  {n->in_d2, nullptr, P1 * 96},
+                   {n->r2, nullptr, P1 * 64},   {n->in_d1, nullptr, P1 * 64},  {n->in_d1, nullptr, P0 * 64},
                    {n->r1, nullptr, P0 * 32},   {n->d1, nullptr, P0 * 32},    {nullptr, n->out, P0 * 16}};
   constexpr int kAct = (int)(sizeof(act) / sizeof(act[0]));
   const size_t lp[kLayers] = {P0, P1, P2, P3, P2, P1, P0, P0};
@@ -859,7 +903,13 @@ AMH_API int amh_net_read(amh_net* n, int32_t which, float* out, int64_t* count) 
   if (*count != (int64_t)src.n) return nfail(n, AMH_EINVAL, "tensor %d has %zu elements, not %lld", which, src.n, (long long)*count);
   const float* dev = src.f;
   if (src.b) {   // BF16 -> FP32 in the scratch buffer (the largest tensor fits)
-    bf16_to_f32_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->gB, src.n);
+    // d3 and d2 exist upsampled only: every other pixel and row of in_d2, in_d1
+    const int sub = which == 10 ? 4 : which == 13 ? 2 : 0;
+    const int C = which == 10 ? 96 : 64;
+    if (sub)
+      subsample_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->gB, n->h2 / sub, n->w2 / sub, C);
+    else
+      bf16_to_f32_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->gB, src.n);
     NTRY(n, cudaGetLastError());
     dev = n->gB;
   }

@@ -225,9 +225,17 @@ enum ConvEpi {
   kEpiPool,     // y16, and up / down: its 2 x 2 mean (H / 2, W / 2)
   kEpiUp,       // y16, and its nearest upsampling (2 H, 2 W)
   kEpiSkip,     // r16 before the skip addition, y16 after
-  kEpiSkipUp    // r16 before the skip addition, the upsampling of the sum
+  kEpiSkipUp,   // r16 before the skip addition, the upsampling of the sum
+  // Data gradients, on to the gradient dy of the layer below (after its ReLU
+  // mask; FP32 and BF16, with its sums over the pixels for the bias gradient):
+  // as separate passes these moved 600 MB and took 170 us of a backward pass at
+  // 800 x 528.
+  kEpiMask,     // raw32 = the gradient; dy = it where mask > 0
+  kEpiDown,     // adjoint of the upsampling: sums of 2 x 2 pixels into raw32 (or null) and dy, (H / 2, W / 2)
+  kEpiSpread    // adjoint of the pooling: add32 + gradient / 4 on 2 x 2 pixels, into dy, (2 H, 2 W)
 };
-__host__ __device__ constexpr bool epi_row_pairs(int epi) { return epi == kEpiPool; }   // tiles come in vertical pairs
+__host__ __device__ constexpr bool epi_row_pairs(int epi) { return epi == kEpiPool || epi == kEpiDown; }   // tiles come in vertical pairs
+__host__ __device__ constexpr bool epi_gradient(int epi) { return epi == kEpiMask || epi == kEpiDown || epi == kEpiSpread; }
 
 struct ConvTcArgs {
   const float* bias;          // Cout or null
@@ -236,6 +244,11 @@ struct ConvTcArgs {
   __nv_bfloat16* r16;         // (H, W, Cout) ReLU output before the skip
   __nv_bfloat16* res16;       // the 2 x 2 mean or the upsampling of the output
   float* y32;                 // (H, W, Cout) FP32 output
+  const __nv_bfloat16* mask;  // data gradients: the ReLU output of the layer below
+  const float* add32;
+  float *raw32, *dy32;
+  __nv_bfloat16* dy16;
+  float* bpart;               // sums of dy per CTA and lane quarter: row 4 blockIdx.x + quarter, Cout channels
   unsigned int* status;       // bit 0: a barrier wait gave up
   int H, W, Cin, Cout, relu;
   int Nb;                     // output channels per CTA (a multiple of 16 dividing Cout, at most kConvMaxNb)
@@ -422,6 +435,24 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
     constexpr bool kSkipIn = kEpi == kEpiSkip || kEpi == kEpiSkipUp;
     uint32_t tc = 0;
     [[maybe_unused]] uint4 plo, phi;      // kEpiPool: the even row's output of this pixel
+    [[maybe_unused]] float prow[16];      // kEpiDown: the even row's gradient
+    [[maybe_unused]] float bsum[16];      // sums of dy over this lane's pixels
+    if constexpr (epi_gradient(kEpi)) {
+#pragma unroll
+      for (int e = 0; e < 16; e++) bsum[e] = 0.f;
+    }
+    // dy of eight channels at offset q, sums from channel e0 on
+    auto emit = [&](float* g, uint4 mask, size_t q, int e0) {
+      float m[8];
+      unpack8(mask, m);
+#pragma unroll
+      for (int e = 0; e < 8; e++) {
+        g[e] = m[e] > 0.f ? g[e] : 0.f;
+        bsum[e0 + e] += g[e];
+      }
+      store8(a.dy32 + q, g);
+      *reinterpret_cast<uint4*>(a.dy16 + q) = pack8(g);
+    };
     TileRun r;
     for (int u = lo; ok && next_run(u, hi, a.H, r);) {
       for (int i = 0; i < r.len && ok; i++, tc++) {
@@ -431,9 +462,18 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
         const size_t o = ((size_t)y * a.W + (in ? px : 0)) * a.Cout + co0 + c0;
         // this lane's skip values, fetched while the tile's MMAs run
         [[maybe_unused]] uint4 sk0, sk1;
-        if (kSkipIn) {
+        if constexpr (kSkipIn) {
           sk0 = __ldg(reinterpret_cast<const uint4*>(a.skip + o));
           sk1 = __ldg(reinterpret_cast<const uint4*>(a.skip + o) + 1);
+        }
+        [[maybe_unused]] size_t oq = 0;       // kEpiDown: this lane's eight channels of the pixel pair
+        if constexpr (kEpi == kEpiMask) {
+          sk0 = __ldg(reinterpret_cast<const uint4*>(a.mask + o));
+          sk1 = __ldg(reinterpret_cast<const uint4*>(a.mask + o) + 1);
+        }
+        if constexpr (kEpi == kEpiDown) {
+          oq = ((size_t)(y >> 1) * (a.W >> 1) + (in ? px >> 1 : 0)) * a.Cout + co0 + c0 + ((lane & 1) ? 8 : 0);
+          if (y & 1) sk0 = __ldg(reinterpret_cast<const uint4*>(a.mask + oq));
         }
         if (!(ok = mbar_wait(&acc_full[b], (tc >> 1) & 1u, 64))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -461,6 +501,56 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
         // Lanes past the row's end compute on their TMEM rows and take part in
         // the exchanges; they store only their partner's pixel.
         const bool odd = (lane & 1) != 0;
+        if constexpr (kEpi == kEpiMask) {
+          if (in) {
+            store8(a.raw32 + o, f);
+            store8(a.raw32 + o + 8, f + 8);
+            emit(f, sk0, o, 0);
+            emit(f + 8, sk1, o + 8, 8);
+          }
+          continue;
+        }
+        if constexpr (kEpi == kEpiDown) {
+          // the even lane sums channels 0-7 of the pair, the odd lane 8-15
+          if (y & 1) {
+            float g[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+              const float r0 = __shfl_xor_sync(0xffffffffu, odd ? prow[e] : prow[8 + e], 1);
+              const float r1 = __shfl_xor_sync(0xffffffffu, odd ? f[e] : f[8 + e], 1);
+              const float x00 = odd ? r0 : prow[e], x01 = odd ? prow[8 + e] : r0;
+              const float x10 = odd ? r1 : f[e], x11 = odd ? f[8 + e] : r1;
+              g[e] = ((x00 + x01) + x10) + x11;
+            }
+            if (in) {
+              if (a.raw32) store8(a.raw32 + oq, g);
+              emit(g, sk0, oq, 0);
+            }
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; e++) prow[e] = f[e];
+          }
+          continue;
+        }
+        if constexpr (kEpi == kEpiSpread) {
+          if (in) {
+#pragma unroll
+            for (int d = 0; d < 4; d++) {
+              const size_t q = ((size_t)(2 * y + (d >> 1)) * (2 * a.W) + 2 * px + (d & 1)) * a.Cout + co0 + c0;
+#pragma unroll
+              for (int h = 0; h < 2; h++) {
+                const uint4 m = __ldg(reinterpret_cast<const uint4*>(a.mask + q) + h);
+                const float4 u0 = __ldg(reinterpret_cast<const float4*>(a.add32 + q) + 2 * h);
+                const float4 u1 = __ldg(reinterpret_cast<const float4*>(a.add32 + q) + 2 * h + 1);
+                float g[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+#pragma unroll
+                for (int e = 0; e < 8; e++) g[e] = g[e] + 0.25f * f[8 * h + e];
+                emit(g, m, q + 8 * h, 8 * h);
+              }
+            }
+          }
+          continue;
+        }
         uint4 h0 = pack8(f), h1 = pack8(f + 8);
         if constexpr (kEpi == kEpiPool) {
           // W and H are even: both pixels and both rows of a pair are inside.
@@ -526,6 +616,19 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
             }
           }
         }
+      }
+    }
+    if constexpr (epi_gradient(kEpi)) {
+      // kEpiDown: even lanes hold channels 0-7, odd lanes 8-15
+      constexpr int kCh = kEpi == kEpiDown ? 8 : 16;
+#pragma unroll
+      for (int e = 0; e < kCh; e++)
+#pragma unroll
+        for (int m = 16; m >= (kEpi == kEpiDown ? 2 : 1); m >>= 1) bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], m);
+      float* d = a.bpart + (size_t)(4 * blockIdx.x + qw) * a.Cout + co0 + c0;
+      if (lane < 16 / kCh) {
+#pragma unroll
+        for (int e = 0; e < kCh; e++) d[kCh * lane + e] = bsum[e];
       }
     }
   }
@@ -635,6 +738,8 @@ __global__ void __launch_bounds__(kThreads) wgrad3x3_tc_kernel(const __grid_cons
     if (lane == 0) {
       const int na = a.stacked ? 3 : (a.Cout + 63) / 64, nbx = (a.Cin + 63) / 64;
       const uint32_t bytes = (uint32_t)na * 128u * (uint32_t)cba + (uint32_t)nbx * 132u * (uint32_t)cbb;
+      pdl_wait();
+      pdl_launch();
       RingPos q{0u, 0u};
       for (int k = 0; k < nk && ok; k++, q = q.next((uint32_t)S)) {
         if (!(ok = mbar_wait(&empty[q.slot], q.phase ^ 1u))) break;
@@ -678,6 +783,7 @@ __global__ void __launch_bounds__(kThreads) wgrad3x3_tc_kernel(const __grid_cons
     // channel l) when stacked, else output channel 32 w + l
     const int g = a.stacked ? warp : dy_cta + 1, co = a.stacked ? lane : warp * 32 + lane;
     const bool rows_used = a.stacked ? warp < 3 : warp * 32 < a.Cout;
+    pdl_wait();
     if (rows_used && (ok = mbar_wait(&acc_full, 0, 64))) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int dx = 0; dx < 3; dx++) {

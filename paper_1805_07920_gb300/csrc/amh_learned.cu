@@ -46,53 +46,27 @@ struct LayerDef { int cin, cout, relu; };
 constexpr LayerDef kNet[kLayers] = {{16, 32, 1}, {32, 64, 1}, {64, 96, 1}, {96, 128, 1},
                                     {128, 96, 1}, {96, 64, 1}, {64, 32, 1}, {32, 16, 0}};
 
-// bias gradient in FP32: db[c] += sum over pixels of dy(p, c), C a multiple
-// of 16 (at most 128), in two passes without atomics.  Pass 1: a thread sums
-// four channels (one float4) of every k-th pixel of its block's range,
-// k = 256 / (C / 4), and the block writes its per-channel sums to part[block].
-// Pass 2: one block per channel adds the partial sums into db.
-constexpr int kBiasBlocks = 2048;     // most pass-1 blocks (rows of the partial sums)
-__global__ void __launch_bounds__(256) bias_grad_kernel(const float* __restrict__ dy, int np, int C,
-                                                        int per_block, float* __restrict__ part) {
-  __shared__ float4 red[256];
-  const int g4 = C >> 2, k = 256 / g4, t = threadIdx.x, g = t % g4, j = t / g4;
-  const int p0 = blockIdx.x * per_block, p1 = min(np, p0 + per_block);
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (j < k) {
-#pragma unroll 4
-    for (int p = p0 + j; p < p1; p += k) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(dy + (size_t)p * C) + g);
-      s.x += v.x;
-      s.y += v.y;
-      s.z += v.z;
-      s.w += v.w;
-    }
-  }
-  red[t] = s;
-  __syncthreads();
-  if (j == 0) {
-    for (int q = 1; q < k; q++) {
-      const float4 v = red[q * g4 + g];
-      s.x += v.x;
-      s.y += v.y;
-      s.z += v.z;
-      s.w += v.w;
-    }
-    reinterpret_cast<float4*>(part + (size_t)blockIdx.x * C)[g] = s;
-  }
-}
-__global__ void __launch_bounds__(256) bias_sum_kernel(const float* __restrict__ part, int nb, int C, float* db) {
+// Bias gradients: db of a layer is the sum of the rows of its partial sums
+// (written by the kernels that produce dy), one block per channel and layer.
+constexpr int kBiasRows = 2048;       // most rows of partial sums of a layer
+struct BiasArgs {
+  const float* part[kLayers];
+  float* db[kLayers];
+  int rows[kLayers], C[kLayers];
+};
+__global__ void __launch_bounds__(256) bias_sum_kernel(BiasArgs a) {
   __shared__ float red[256];
-  const int c = blockIdx.x;
+  const int c = blockIdx.x, L = blockIdx.y, C = a.C[L];
+  if (c >= C) return;
   float s = 0.f;
-  for (int b = threadIdx.x; b < nb; b += 256) s += part[(size_t)b * C + c];
+  for (int b = threadIdx.x; b < a.rows[L]; b += 256) s += a.part[L][(size_t)b * C + c];
   red[threadIdx.x] = s;
   __syncthreads();
   for (int w = 128; w > 0; w >>= 1) {
     if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) db[c] += red[0];
+  if (threadIdx.x == 0) a.db[L][c] = red[0];
 }
 
 // weights (9, Cout, Cin) -> data-gradient weights (9, Cin, Cout), taps flipped
@@ -104,56 +78,6 @@ __global__ void flip_transpose_kernel(const __nv_bfloat16* w, __nv_bfloat16* wd,
   }
 }
 
-// The elementwise kernels below take four channels per thread and step (C is
-// a multiple of 16, so a group of four never crosses a pixel): 16-byte FP32
-// and 8-byte BF16 accesses.
-struct bf16x4 { __nv_bfloat162 a, b; };
-__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
-  const bf16x4 v = *reinterpret_cast<const bf16x4*>(p);
-  const float2 lo = __bfloat1622float2(v.a), hi = __bfloat1622float2(v.b);
-  return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-__device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
-  bf16x4 o;
-  o.a = __floats2bfloat162_rn(v.x, v.y);
-  o.b = __floats2bfloat162_rn(v.z, v.w);
-  *reinterpret_cast<bf16x4*>(p) = o;
-}
-__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-__device__ __forceinline__ float4 scale4(float s, float4 a) { return make_float4(s * a.x, s * a.y, s * a.z, s * a.w); }
-
-__global__ void pool2_bwd_add_kernel(const float* __restrict__ d, float* __restrict__ dx, int H, int W, int C) {   // dx += pool'^T d
-  const size_t n = (size_t)H * W * C / 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(4 * i % C), p = (int)(4 * i / C), yy = p / W, xx = p % W;
-    float4* o = reinterpret_cast<float4*>(dx) + i;
-    *o = add4(*o, scale4(0.25f, *reinterpret_cast<const float4*>(d + ((size_t)(yy / 2) * (W / 2) + xx / 2) * C + c)));
-  }
-}
-__global__ void up2_bwd_kernel(const float* __restrict__ d, float* __restrict__ dx, int H, int W, int C) {   // (H, W) = input size
-  const size_t n = (size_t)H * W * C / 4;
-  const int Wo = 2 * W;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(4 * i % C), p = (int)(4 * i / C), yy = p / W, xx = p % W;
-    const float* b = d + ((size_t)(2 * yy) * Wo + 2 * xx) * C + c;
-    const float4 s = add4(add4(add4(*reinterpret_cast<const float4*>(b), *reinterpret_cast<const float4*>(b + C)),
-                               *reinterpret_cast<const float4*>(b + (size_t)Wo * C)),
-                          *reinterpret_cast<const float4*>(b + (size_t)Wo * C + C));
-    reinterpret_cast<float4*>(dx)[i] = s;
-  }
-}
-// g (FP32) times the ReLU mask of r, optionally also into a BF16 copy; n a
-// multiple of 4
-__global__ void relu_mask_kernel(const float* __restrict__ g, const __nv_bfloat16* __restrict__ r, float* __restrict__ out,
-                                 __nv_bfloat16* __restrict__ out16, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 gv = reinterpret_cast<const float4*>(g)[i], rv = ld4(r + 4 * i);
-    const float4 v = make_float4(rv.x > 0.f ? gv.x : 0.f, rv.y > 0.f ? gv.y : 0.f, rv.z > 0.f ? gv.z : 0.f,
-                                 rv.w > 0.f ? gv.w : 0.f);
-    reinterpret_cast<float4*>(out)[i] = v;
-    if (out16) st4(out16 + 4 * i, v);
-  }
-}
 __global__ void bf16_to_f32_kernel(const __nv_bfloat16* g, float* o, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     o[i] = __bfloat162float(g[i]);
@@ -171,13 +95,30 @@ __global__ void to_bf16_kernel(const float* g, __nv_bfloat16* o, size_t n) {
     o[i] = __float2bfloat16(g[i]);
 }
 
-// L1 loss over the 4 used output channels of the masked pixels and its
-// gradient (zero on the other 12 channels); loss accumulated in *loss (sum;
-// the host divides by the count)
-__global__ void l1_loss_kernel(const float* __restrict__ out, const float* __restrict__ target,
-                               const uint8_t* __restrict__ mask, float* __restrict__ dout, float* loss, int np,
-                               float inv_n) {
-  float s = 0.f;
+// sum of the mask's bytes into *count (zeroed before)
+__global__ void __launch_bounds__(256) mask_count_kernel(const uint8_t* __restrict__ mask, int np, unsigned int* count) {
+  unsigned int s = 0;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < np / 16; i += gridDim.x * 256) {
+    const uint4 v = reinterpret_cast<const uint4*>(mask)[i];   // np is a multiple of 64
+    s = __dp4a(v.x, 0x01010101u, s);
+    s = __dp4a(v.y, 0x01010101u, s);
+    s = __dp4a(v.z, 0x01010101u, s);
+    s = __dp4a(v.w, 0x01010101u, s);
+  }
+  s = __reduce_add_sync(0xffffffffu, s);
+  if ((threadIdx.x & 31) == 0 && s) atomicAdd(count, s);
+}
+// L1 loss over the 4 used output channels of the masked pixels, divided by the
+// mask's sum, and its gradient (zero on the other 12 channels) in FP32 and
+// BF16, with its sums per block for the bias gradient; the loss goes to *loss
+// (zeroed before), one addition per block
+__global__ void __launch_bounds__(256) l1_loss_kernel(const float* __restrict__ out, const float* __restrict__ target,
+                                                      const uint8_t* __restrict__ mask,
+                                                      const unsigned int* __restrict__ count, float* __restrict__ dout,
+                                                      __nv_bfloat16* __restrict__ dout16, float* __restrict__ part,
+                                                      float* loss, int np) {
+  const float inv_n = 1.f / (float)max(1u, *count);
+  float s = 0.f, gs[4] = {0.f, 0.f, 0.f, 0.f};
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const float4 o = reinterpret_cast<const float4*>(out)[(size_t)p * 4];
     const float4 t = reinterpret_cast<const float4*>(target)[p];
@@ -191,25 +132,70 @@ __global__ void l1_loss_kernel(const float* __restrict__ out, const float* __res
         s += fabsf(d[c]);
         g[c] = (d[c] > 0.f ? 1.f : (d[c] < 0.f ? -1.f : 0.f)) * inv_n;
       }
+      gs[c] += g[c];
     }
     float4* dp = reinterpret_cast<float4*>(dout) + (size_t)p * 4;
     dp[0] = make_float4(g[0], g[1], g[2], g[3]);
     dp[1] = dp[2] = dp[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint4* dh = reinterpret_cast<uint4*>(dout16) + (size_t)p * 2;
+    dh[0] = make_uint4(tc::pack_bf16(g[0], g[1]), tc::pack_bf16(g[2], g[3]), 0u, 0u);
+    dh[1] = make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv_n);
+  __shared__ float red[8][5];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+    for (int c = 0; c < 4; c++) gs[c] += __shfl_xor_sync(0xffffffffu, gs[c], o);
+  }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[warp][4] = s;
+    for (int c = 0; c < 4; c++) red[warp][c] = gs[c];
+  }
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    float v = 0.f;
+    if (threadIdx.x < 4)
+      for (int w = 0; w < 8; w++) v += red[w][threadIdx.x];
+    part[(size_t)blockIdx.x * 16 + threadIdx.x] = v;
+  }
+  if (threadIdx.x == 32) {
+    float v = 0.f;
+    for (int w = 0; w < 8; w++) v += red[w][4];
+    atomicAdd(loss, v * inv_n);
+  }
 }
 
-__global__ void adam_kernel(float* w, float* m, float* v, const float* g, __nv_bfloat16* w16, int n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    if (w16) w16[i] = __float2bfloat16(wi);
+// One Adam step of every layer (the layers' weights lie one after another, then
+// their biases), the weights' BF16 copy and its flipped transpose for the data
+// gradients (flip_transpose_kernel).
+struct AdamArgs {
+  float *w, *m, *v;
+  const float* g;
+  __nv_bfloat16 *w16, *wd16;
+  int n_weights, n;
+  int start[kLayers], cin[kLayers], cout[kLayers];
+  float lr, b1, b2, eps, c1, c2;
+};
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamArgs a) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
+    const float gi = a.g[i];
+    const float mi = a.b1 * a.m[i] + (1.f - a.b1) * gi, vi = a.b2 * a.v[i] + (1.f - a.b2) * gi * gi;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float wi = a.w[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    a.w[i] = wi;
+    if (i < a.n_weights) {
+      int L = 0;
+#pragma unroll
+      for (int l = 1; l < kLayers; l++) L += i >= a.start[l];
+      const int q = i - a.start[L], cin = a.cin[L], cout = a.cout[L];
+      const int ci = q % cin, co = q / cin % cout, t = q / (cin * cout);
+      const __nv_bfloat16 h = __float2bfloat16(wi);
+      a.w16[i] = h;
+      a.wd16[a.start[L] + ((8 - t) * cin + ci) * cout + co] = h;
+    }
   }
 }
 
@@ -334,25 +320,33 @@ struct amh_net {
   __nv_bfloat16* wd16[kLayers] = {};      // data-gradient weights
   float *mw[kLayers] = {}, *vw[kLayers] = {}, *mb[kLayers] = {}, *vb[kLayers] = {};
   float *gw[kLayers] = {}, *gb[kLayers] = {};
-  float* bpart = nullptr;                 // per-block partial sums of the bias gradients
+  // the layers' arrays lie one after another (weights, then biases): wm, mw,
+  // vw and gw of layer 0 start the whole; the loss and the mask's sum follow the
+  // gradients
+  size_t n_weights = 0, n_params = 0;
+  float* bpart[kLayers] = {};             // partial sums of the bias gradients
+  int brows[kLayers] = {};                // and their rows
   int step = 0;
   // activations (BF16) and gradient buffers (FP32)
   __nv_bfloat16 *x0 = nullptr, *e1 = nullptr, *in_e2 = nullptr, *e2 = nullptr, *in_e3 = nullptr, *e3 = nullptr,
                 *in_e4 = nullptr, *e4 = nullptr, *in_d3 = nullptr, *r3 = nullptr, *in_d2 = nullptr,
-                *r2 = nullptr, *in_d1 = nullptr, *r1 = nullptr, *d1 = nullptr, *g16 = nullptr;
+                *r2 = nullptr, *in_d1 = nullptr, *r1 = nullptr, *d1 = nullptr;
   float* out = nullptr;
   float* target = nullptr;
   uint8_t* mask = nullptr;
   float4* pin = nullptr;
   float4* prop = nullptr;
-  // backward: dy[L] = gradient at layer L's output after its ReLU mask (FP32),
-  // gA / gB scratch, gE1..gE3 gradients arriving at e1..e3 through the skips
+  // backward: dy[L] = gradient at layer L's output after its ReLU mask (FP32,
+  // and a BF16 copy the tensor cores read), gE1..gE3 gradients arriving at
+  // e1..e3 through the skips
   float* dy[kLayers] = {};
-  float *gA = nullptr, *gB = nullptr, *gE1 = nullptr, *gE2 = nullptr, *gE3 = nullptr;
+  __nv_bfloat16* dy16[kLayers] = {};
+  float *gE1 = nullptr, *gE2 = nullptr, *gE3 = nullptr;
+  float* scratch = nullptr;               // 64 floats per pixel: host examples, tensors read back
   ConvOp fwd[kLayers], dgr[kLayers];      // forward; data gradients (layer 0 has none)
   float* loss = nullptr;
+  unsigned int* count = nullptr;          // sum of the mask
   unsigned int* status = nullptr;         // bit 0: a convolution's barrier wait gave up
-  size_t maxel = 0;
   std::vector<void*> allocs;
   std::string err;
 };
@@ -426,6 +420,9 @@ const void* conv_kernel(int epi) {
     case tc::kEpiUp: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiUp>);
     case tc::kEpiSkip: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiSkip>);
     case tc::kEpiSkipUp: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiSkipUp>);
+    case tc::kEpiMask: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiMask>);
+    case tc::kEpiDown: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiDown>);
+    case tc::kEpiSpread: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiSpread>);
     default: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiPlain>);
   }
 }
@@ -491,10 +488,10 @@ int plan_conv(amh_net* n, ConvOp& op, const __nv_bfloat16* x, const __nv_bfloat1
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "conv: kernel attributes: %s", cudaGetErrorString(e));
   // persistent grid: per channel block, as many CTAs as fit on the SMs at
   // once (every CTA holds its tensor memory until it exits), by the plan and by
-  // the register file; at most one per tile
+  // the register file; at most one per tile (or pair of tiles)
   const int by_regs = 65536 / (((fa.numRegs + 7) & ~7) * op.threads);
   const int cps = std::max(1, std::min(p.ctas_per_sm, by_regs));
-  const int nblk = Cout / p.Nb, ntiles = H * ((W + tc::kM - 1) / tc::kM);
+  const int nblk = Cout / p.Nb, ntiles = H * ((W + tc::kM - 1) / tc::kM) / (tc::epi_row_pairs(epi) ? 2 : 1);
   op.grid = dim3(std::max(1, std::min(ntiles, n_sm * cps / nblk)), nblk);
   return AMH_OK;
 }
@@ -534,20 +531,43 @@ int plan_network(amh_net* n) {
     a.relu = kNet[L].relu;
     rc = plan_conv(n, n->fwd[L], f[L].x, n->w16[L], f[L].H, f[L].W, kNet[L].cin, kNet[L].cout, f[L].epi, a);
   }
-  // data gradients: dx (FP32, H x W x Cin, in gA) from dy (BF16 copy in g16)
+  // data gradients, from dy16[L] to dy[L - 1] (or, through the pooling and the
+  // skips, to the layer the gradient passes on to)
+  struct D {
+    int epi, to;
+    const __nv_bfloat16* mask;
+    const float* add;
+    float* raw;
+  };
+  const D d[kLayers] = {{},
+                        {tc::kEpiSpread, 0, n->e1, n->gE1, nullptr},
+                        {tc::kEpiSpread, 1, n->e2, n->gE2, nullptr},
+                        {tc::kEpiSpread, 2, n->e3, n->gE3, nullptr},
+                        {tc::kEpiDown, 3, n->e4, nullptr, nullptr},      // in_d3 = up(e4)
+                        {tc::kEpiDown, 4, n->r3, nullptr, n->gE3},       // in_d2 = up(d3), d3 = r3 + e3
+                        {tc::kEpiDown, 5, n->r2, nullptr, n->gE2},       // in_d1 = up(d2), d2 = r2 + e2
+                        {tc::kEpiMask, 6, n->r1, nullptr, n->gE1}};      // d1 = r1 + e1
   for (int L = 1; L < kLayers && !rc; L++) {
     tc::ConvTcArgs a{};
-    a.y32 = n->gA;
-    rc = plan_conv(n, n->dgr[L], n->g16, n->wd16[L], f[L].H, f[L].W, kNet[L].cout, kNet[L].cin, tc::kEpiPlain, a);
+    a.mask = d[L].mask;
+    a.add32 = d[L].add;
+    a.raw32 = d[L].raw;
+    a.dy32 = n->dy[d[L].to];
+    a.dy16 = n->dy16[d[L].to];
+    a.bpart = n->bpart[d[L].to];
+    rc = plan_conv(n, n->dgr[L], n->dy16[L], n->wd16[L], f[L].H, f[L].W, kNet[L].cout, kNet[L].cin, d[L].epi, a);
+    n->brows[d[L].to] = 4 * (int)n->dgr[L].grid.x;
+    if (!rc && n->brows[d[L].to] > kBiasRows) rc = nfail(n, AMH_EINVAL, "conv: more partial sums than rows");
   }
   return rc;
 }
-// weight gradient of layer L from its input x and its output gradient (FP32
-// dy for the bias, its BF16 copy dy16 for the weights): the tensor-core
-// kernel reads both pixel-major and sums a band of rows per CTA (all nine
-// taps when Cout <= 32, else the three of one vertical tap) into gw
-int wgrad(amh_net* n, int L, const __nv_bfloat16* x, const float* dy, const __nv_bfloat16* dy16, int H, int W) {
-  const int Cin = kNet[L].cin, Cout = kNet[L].cout, np = H * W;
+// weight gradient of layer L from its input x and its output gradient (BF16
+// dy16): the tensor-core kernel reads both pixel-major and sums a band of rows
+// per CTA (all nine taps when Cout <= 32, else the three of one vertical tap)
+// into gw
+int wgrad(amh_net* n, int L, const __nv_bfloat16* x, int H, int W) {
+  const int Cin = kNet[L].cin, Cout = kNet[L].cout;
+  const __nv_bfloat16* dy16 = n->dy16[L];
   const int stacked = Cout <= 32 ? 1 : 0, cba = stacked ? Cout : 64, cbb = tc::wgrad_xbox(Cin);
   CUtensorMap mdy, mx;
   if (!bf16_map(&mdy, dy16, Cout, W, H, cba, 64, 1, 0, block_swizzle(cba)) ||
@@ -573,12 +593,6 @@ int wgrad(amh_net* n, int L, const __nv_bfloat16* x, const float* dy, const __nv
   const int per_cta = (steps + std::max(1, n_sm / gy) - 1) / std::max(1, n_sm / gy);
   const tc::WgradTcArgs a{n->gw[L], n->status, H, W, Cin, Cout, per_cta, stacked, S};
   tc::wgrad3x3_tc_kernel<<<dim3((steps + per_cta - 1) / per_cta, gy), tc::kThreads, smem, n->stream>>>(mdy, mx, a);
-  // about eight blocks per SM (at most kBiasBlocks), each a whole number of
-  // the block's pixel steps
-  const int step = 256 / (Cout / 4), want = std::min(kBiasBlocks, 8 * n_sm), per = (np + want - 1) / want;
-  const int per_block = std::max(step, (per + step - 1) / step * step), nb = (np + per_block - 1) / per_block;
-  bias_grad_kernel<<<nb, 256, 0, n->stream>>>(dy, np, Cout, per_block, n->bpart);
-  bias_sum_kernel<<<Cout, 256, 0, n->stream>>>(n->bpart, nb, Cout, n->gb[L]);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "wgrad launch: %s", cudaGetErrorString(e));
   return AMH_OK;
@@ -619,32 +633,48 @@ AMH_API int amh_net_create(amh_net** out, int32_t width2, int32_t height2, uint6
     s = s * 6364136223846793005ull + 1442695040888963407ull;
     return ((s >> 11) + 0.5) * (1.0 / 9007199254740992.0);
   };
+  for (const LayerDef& d : kNet) {
+    n->n_weights += (size_t)9 * d.cin * d.cout;
+    n->n_params += (size_t)9 * d.cin * d.cout + d.cout;
+  }
+  float *pw, *pm, *pv, *pg;
+  __nv_bfloat16 *p16, *pd16;
+  NA(pw, n->n_params); NA(pm, n->n_params); NA(pv, n->n_params); NA(pg, n->n_params + 2);
+  NA(p16, n->n_weights); NA(pd16, n->n_weights);
+  n->loss = pg + n->n_params;
+  n->count = reinterpret_cast<unsigned int*>(n->loss + 1);
+  size_t ow = 0, ob = n->n_weights;
   for (int L = 0; L < kLayers; L++) {
     const int Cin = kNet[L].cin, Cout = kNet[L].cout;
     const size_t nw = (size_t)9 * Cin * Cout;
-    NA(n->wm[L], nw); NA(n->w16[L], nw); NA(n->wd16[L], nw); NA(n->mw[L], nw); NA(n->vw[L], nw); NA(n->gw[L], nw);
-    NA(n->bm[L], Cout); NA(n->mb[L], Cout); NA(n->vb[L], Cout); NA(n->gb[L], Cout);
+    n->wm[L] = pw + ow; n->mw[L] = pm + ow; n->vw[L] = pv + ow; n->gw[L] = pg + ow;
+    n->w16[L] = p16 + ow; n->wd16[L] = pd16 + ow;
+    n->bm[L] = pw + ob; n->mb[L] = pm + ob; n->vb[L] = pv + ob; n->gb[L] = pg + ob;
+    ow += nw;
+    ob += Cout;
+    NA(n->bpart[L], (size_t)kBiasRows * Cout);
     std::vector<float> w(nw);
     const double sd = std::sqrt(2.0 / (9.0 * Cin)) * (L == kLayers - 1 ? 0.1 : 1.0);
     for (size_t i = 0; i < nw; i++) w[i] = (float)(sd * std::sqrt(-2.0 * std::log(uni())) * std::cos(6.283185307179586 * uni()));
     cudaMemcpyAsync(n->wm[L], w.data(), nw * sizeof(float), cudaMemcpyHostToDevice, n->stream);
     cudaStreamSynchronize(n->stream);
   }
-  NA(n->bpart, (size_t)kBiasBlocks * 128);
   NA(n->status, 1);
   const size_t P0 = (size_t)width2 * height2, P1 = P0 / 4, P2 = P0 / 16, P3 = P0 / 64;
   NA(n->x0, P0 * 16); NA(n->e1, P0 * 32); NA(n->in_e2, P1 * 32); NA(n->e2, P1 * 64); NA(n->in_e3, P2 * 64);
   NA(n->e3, P2 * 96); NA(n->in_e4, P3 * 96); NA(n->e4, P3 * 128); NA(n->in_d3, P2 * 128); NA(n->r3, P2 * 96);
   NA(n->in_d2, P1 * 96); NA(n->r2, P1 * 64); NA(n->in_d1, P0 * 64);
   NA(n->r1, P0 * 32); NA(n->d1, P0 * 32);
-  n->maxel = P0 * 64;
-  NA(n->g16, n->maxel); NA(n->gA, n->maxel); NA(n->gB, n->maxel);
+  NA(n->scratch, P0 * 64);
   {
     const size_t lp[kLayers] = {P0, P1, P2, P3, P2, P1, P0, P0};   // output size of each layer
-    for (int L = 0; L < kLayers; L++) NA(n->dy[L], lp[L] * kNet[L].cout);
+    for (int L = 0; L < kLayers; L++) {
+      NA(n->dy[L], lp[L] * kNet[L].cout);
+      NA(n->dy16[L], lp[L] * kNet[L].cout);
+    }
   }
   NA(n->gE1, P0 * 32); NA(n->gE2, P1 * 64); NA(n->gE3, P2 * 96);
-  NA(n->out, P0 * 16); NA(n->target, P0 * 4); NA(n->mask, P0); NA(n->pin, P0); NA(n->prop, P0); NA(n->loss, 1);
+  NA(n->out, P0 * 16); NA(n->target, P0 * 4); NA(n->mask, P0); NA(n->pin, P0); NA(n->prop, P0);
 #undef NA
   if (const int rc = plan_network(n)) return bail(rc);
   for (int L = 0; L < kLayers; L++) {
@@ -706,18 +736,20 @@ AMH_API int amh_net_set_example(amh_net* n, const float* x, int32_t channels, co
   const size_t np = (size_t)n->w2 * n->h2;
   const float *dx = x, *dt = target;
   const uint8_t* dm = mask;
-  if (mem == AMH_MEM_HOST) {   // into the scratch buffers (gA: features, gB: targets, then the mask)
-    NTRY(n, cudaMemcpyAsync(n->gA, x, np * channels * 4, cudaMemcpyHostToDevice, n->stream));
-    NTRY(n, cudaMemcpyAsync(n->gB, target, np * 16, cudaMemcpyHostToDevice, n->stream));
-    uint8_t* mb = reinterpret_cast<uint8_t*>(n->gB + np * 4);
-    NTRY(n, cudaMemcpyAsync(mb, mask, np, cudaMemcpyHostToDevice, n->stream));
-    dx = n->gA;
-    dt = n->gB;
-    dm = mb;
+  float* const ts = n->scratch;           // targets, then the features, then the mask
+  if (mem == AMH_MEM_HOST) {
+    float* xs = ts + np * 4;
+    uint8_t* ms = reinterpret_cast<uint8_t*>(xs + np * 16);
+    NTRY(n, cudaMemcpyAsync(xs, x, np * channels * 4, cudaMemcpyHostToDevice, n->stream));
+    NTRY(n, cudaMemcpyAsync(ts, target, np * 16, cudaMemcpyHostToDevice, n->stream));
+    NTRY(n, cudaMemcpyAsync(ms, mask, np, cudaMemcpyHostToDevice, n->stream));
+    dx = xs;
+    dt = ts;
+    dm = ms;
   }
   if (reinterpret_cast<uintptr_t>(dt) & 15) {   // the kernel reads each pixel's targets as one float4
-    NTRY(n, cudaMemcpyAsync(n->gB, dt, np * 16, cudaMemcpyDeviceToDevice, n->stream));
-    dt = n->gB;
+    NTRY(n, cudaMemcpyAsync(ts, dt, np * 16, cudaMemcpyDeviceToDevice, n->stream));
+    dt = ts;
   }
   example_kernel<<<blocks_for(np), 256, 0, n->stream>>>(dx, channels, dt, dm, n->w2, n->h2, mirror & 3, n->x0,
                                                         n->target, n->mask);
@@ -771,57 +803,28 @@ AMH_API int amh_net_forward(amh_net* n, float* out_host) {
 // loss of the last forward against the targets, and all gradients
 AMH_API int amh_net_backward(amh_net* n, float* loss_out) {
   if (!n) return AMH_EINVAL;
-  const int W0 = n->w2, H0 = n->h2, W1 = W0 / 2, H1 = H0 / 2, W2 = W1 / 2, H2 = H1 / 2, W3 = W2 / 2, H3 = H2 / 2;
-  const size_t P0 = (size_t)W0 * H0, P1 = P0 / 4, P2 = P0 / 16, P3 = P0 / 64;
+  const size_t P0 = (size_t)n->w2 * n->h2;
   const cudaStream_t s = n->stream;
-  // mask count on the host side of the stream
-  std::vector<uint8_t> mk(P0);
-  NTRY(n, cudaMemcpyAsync(mk.data(), n->mask, P0, cudaMemcpyDeviceToHost, s));
-  NTRY(n, cudaStreamSynchronize(s));
-  size_t cnt = 0;
-  for (uint8_t m : mk) cnt += m;
-  const float inv_n = 1.f / (float)std::max<size_t>(1, cnt);
-  for (int L = 0; L < kLayers; L++) {
-    NTRY(n, cudaMemsetAsync(n->gw[L], 0, (size_t)9 * kNet[L].cin * kNet[L].cout * 4, s));
-    NTRY(n, cudaMemsetAsync(n->gb[L], 0, (size_t)kNet[L].cout * 4, s));
+  // gradients, loss and the mask's sum
+  NTRY(n, cudaMemsetAsync(n->gw[0], 0, (n->n_params + 2) * sizeof(float), s));
+  mask_count_kernel<<<(int)std::min<size_t>((P0 / 16 + 255) / 256, 152), 256, 0, s>>>(n->mask, (int)P0, n->count);
+  const int lb = (int)std::min<size_t>((P0 + 255) / 256, kBiasRows);
+  l1_loss_kernel<<<lb, 256, 0, s>>>(n->out, n->target, n->mask, n->count, n->dy[7], n->dy16[7], n->bpart[7], n->loss, (int)P0);
+  n->brows[7] = lb;
+  const __nv_bfloat16* x[kLayers] = {n->x0, n->in_e2, n->in_e3, n->in_e4, n->in_d3, n->in_d2, n->in_d1, n->d1};
+  int rc = AMH_OK;
+  for (int L = kLayers - 1; L >= 0 && !rc; L--) {
+    rc = wgrad(n, L, x[L], n->fwd[L].a.H, n->fwd[L].a.W);
+    if (!rc && L > 0) rc = conv(n, n->dgr[L], true);
   }
-  NTRY(n, cudaMemsetAsync(n->loss, 0, 4, s));
-  float* const* dy = n->dy;
-  l1_loss_kernel<<<blocks_for(P0), 256, 0, s>>>(n->out, n->target, n->mask, dy[7], n->loss, (int)P0, inv_n);
-  // out = conv(d1)
-  to_bf16_kernel<<<blocks_for(P0 * 16), 256, 0, s>>>(dy[7], n->g16, P0 * 16);
-  int rc = wgrad(n, 7, n->d1, dy[7], n->g16, H0, W0);
-  if (!rc) rc = conv(n, n->dgr[7], false);                  // gA = d d1 (P0 x 32)
-  // d1 = relu(conv(in_d1)) + e1
-  NTRY(n, cudaMemcpyAsync(n->gE1, n->gA, P0 * 32 * 4, cudaMemcpyDeviceToDevice, s));
-  relu_mask_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gA, n->r1, dy[6], n->g16, P0 * 32);
-  if (!rc) rc = wgrad(n, 6, n->in_d1, dy[6], n->g16, H0, W0);
-  if (!rc) rc = conv(n, n->dgr[6], false);                  // d in_d1 (P0 x 64)
-  up2_bwd_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gA, n->gE2, H1, W1, 64);  // d d2 (P1 x 64)
-  relu_mask_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gE2, n->r2, dy[5], n->g16, P1 * 64);
-  if (!rc) rc = wgrad(n, 5, n->in_d2, dy[5], n->g16, H1, W1);
-  if (!rc) rc = conv(n, n->dgr[5], false);                  // d in_d2 (P1 x 96)
-  up2_bwd_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gA, n->gE3, H2, W2, 96);  // d d3 (P2 x 96)
-  relu_mask_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gE3, n->r3, dy[4], n->g16, P2 * 96);
-  if (!rc) rc = wgrad(n, 4, n->in_d3, dy[4], n->g16, H2, W2);
-  if (!rc) rc = conv(n, n->dgr[4], false);                  // d in_d3 (P2 x 128)
-  up2_bwd_kernel<<<blocks_for(P3 * 128), 256, 0, s>>>(n->gA, n->gB, H3, W3, 128); // d e4 (P3 x 128)
-  // e4 = relu(conv(in_e4))
-  relu_mask_kernel<<<blocks_for(P3 * 128), 256, 0, s>>>(n->gB, n->e4, dy[3], n->g16, P3 * 128);
-  if (!rc) rc = wgrad(n, 3, n->in_e4, dy[3], n->g16, H3, W3);
-  if (!rc) rc = conv(n, n->dgr[3], false);                  // d in_e4 (P3 x 96)
-  pool2_bwd_add_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gA, n->gE3, H2, W2, 96);
-  // e3 = relu(conv(in_e3)), read by d3 (skip) and by the pooling
-  relu_mask_kernel<<<blocks_for(P2 * 96), 256, 0, s>>>(n->gE3, n->e3, dy[2], n->g16, P2 * 96);
-  if (!rc) rc = wgrad(n, 2, n->in_e3, dy[2], n->g16, H2, W2);
-  if (!rc) rc = conv(n, n->dgr[2], false);                  // d in_e3 (P2 x 64)
-  pool2_bwd_add_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gA, n->gE2, H1, W1, 64);
-  relu_mask_kernel<<<blocks_for(P1 * 64), 256, 0, s>>>(n->gE2, n->e2, dy[1], n->g16, P1 * 64);
-  if (!rc) rc = wgrad(n, 1, n->in_e2, dy[1], n->g16, H1, W1);
-  if (!rc) rc = conv(n, n->dgr[1], false);                  // d in_e2 (P1 x 32)
-  pool2_bwd_add_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gA, n->gE1, H0, W0, 32);
-  relu_mask_kernel<<<blocks_for(P0 * 32), 256, 0, s>>>(n->gE1, n->e1, dy[0], n->g16, P0 * 32);
-  if (!rc) rc = wgrad(n, 0, n->x0, dy[0], n->g16, H0, W0);
+  BiasArgs ba;
+  for (int L = 0; L < kLayers; L++) {
+    ba.part[L] = n->bpart[L];
+    ba.db[L] = n->gb[L];
+    ba.rows[L] = n->brows[L];
+    ba.C[L] = kNet[L].cout;
+  }
+  bias_sum_kernel<<<dim3(128, kLayers), 256, 0, s>>>(ba);
   if (rc) return rc;
   NTRY(n, cudaGetLastError());
   if (loss_out) {
@@ -836,14 +839,27 @@ AMH_API int amh_net_adam(amh_net* n, float lr) {
   n->step++;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)n->step), c2 = 1.f - std::pow(b2, (float)n->step);
+  AdamArgs a;
+  a.w = n->wm[0];
+  a.m = n->mw[0];
+  a.v = n->vw[0];
+  a.g = n->gw[0];
+  a.w16 = n->w16[0];
+  a.wd16 = n->wd16[0];
+  a.n_weights = (int)n->n_weights;
+  a.n = (int)n->n_params;
   for (int L = 0; L < kLayers; L++) {
-    const size_t nw = (size_t)9 * kNet[L].cin * kNet[L].cout;
-    adam_kernel<<<blocks_for(nw), 256, 0, n->stream>>>(n->wm[L], n->mw[L], n->vw[L], n->gw[L], n->w16[L], (int)nw,
-                                                     lr, b1, b2, 1e-8f, c1, c2);
-    adam_kernel<<<1, 256, 0, n->stream>>>(n->bm[L], n->mb[L], n->vb[L], n->gb[L], nullptr, kNet[L].cout, lr, b1, b2,
-                                         1e-8f, c1, c2);
-    flip_transpose_kernel<<<blocks_for(nw), 256, 0, n->stream>>>(n->w16[L], n->wd16[L], kNet[L].cin, kNet[L].cout);
+    a.start[L] = (int)(n->wm[L] - n->wm[0]);
+    a.cin[L] = kNet[L].cin;
+    a.cout[L] = kNet[L].cout;
   }
+  a.lr = lr;
+  a.b1 = b1;
+  a.b2 = b2;
+  a.eps = 1e-8f;
+  a.c1 = c1;
+  a.c2 = c2;
+  adam_kernel<<<blocks_for(n->n_params), 256, 0, n->stream>>>(a);
   NTRY(n, cudaGetLastError());
   return AMH_OK;
 }
@@ -907,11 +923,11 @@ AMH_API int amh_net_read(amh_net* n, int32_t which, float* out, int64_t* count) 
     const int sub = which == 10 ? 4 : which == 13 ? 2 : 0;
     const int C = which == 10 ? 96 : 64;
     if (sub)
-      subsample_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->gB, n->h2 / sub, n->w2 / sub, C);
+      subsample_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->scratch, n->h2 / sub, n->w2 / sub, C);
     else
-      bf16_to_f32_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->gB, src.n);
+      bf16_to_f32_kernel<<<blocks_for(src.n), 256, 0, n->stream>>>(src.b, n->scratch, src.n);
     NTRY(n, cudaGetLastError());
-    dev = n->gB;
+    dev = n->scratch;
   }
   NTRY(n, cudaMemcpyAsync(out, dev, src.n * 4, cudaMemcpyDeviceToHost, n->stream));
   NTRY(n, cudaStreamSynchronize(n->stream));

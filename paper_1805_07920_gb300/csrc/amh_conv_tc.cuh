@@ -184,9 +184,28 @@ __device__ __forceinline__ void unpack8(uint4 v, float* f) {
   const float2 a = unpack_bf16(v.x), b = unpack_bf16(v.y), c = unpack_bf16(v.z), d = unpack_bf16(v.w);
   f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y; f[4] = c.x; f[5] = c.y; f[6] = d.x; f[7] = d.y;
 }
-__device__ __forceinline__ void store8(float* p, const float* f) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(f[0], f[1], f[2], f[3]);
-  reinterpret_cast<float4*>(p)[1] = make_float4(f[4], f[5], f[6], f[7]);
+// Transpose within each group of four lanes (four neighbouring pixels, 16 FP32
+// channels each): t[k] becomes channels 4 (lane % 4) .. + 3 of pixel k of the
+// group, so that one 16-byte access per lane covers 64 contiguous bytes of
+// eight pixels instead of 16 bytes of 32.  All 32 lanes call it.
+__device__ __forceinline__ void quad_transpose(float (&t)[4][4], int lane) {
+#pragma unroll
+  for (int s = 1; s <= 2; s <<= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (k & s) continue;
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const float r = __shfl_xor_sync(0xffffffffu, up ? t[k][e] : t[k + s][e], s);
+        if (up) t[k][e] = r;
+        else t[k + s][e] = r;
+      }
+    }
+  }
+}
+__device__ __forceinline__ void store4(float* p, const float* f) {
+  *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
 }
 
 // Forward / data-gradient kernel.  A tile is 128 consecutive pixels of one
@@ -435,23 +454,20 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
     constexpr bool kSkipIn = kEpi == kEpiSkip || kEpi == kEpiSkipUp;
     uint32_t tc = 0;
     [[maybe_unused]] uint4 plo, phi;      // kEpiPool: the even row's output of this pixel
-    [[maybe_unused]] float prow[16];      // kEpiDown: the even row's gradient
-    [[maybe_unused]] float bsum[16];      // sums of dy over this lane's pixels
-    if constexpr (epi_gradient(kEpi)) {
+    [[maybe_unused]] float prow[4][4];    // kEpiDown: the even row's gradient (quad_transpose)
+    [[maybe_unused]] float bsum[4] = {0.f, 0.f, 0.f, 0.f};   // sums of dy, channels 4 (lane % 4) .. + 3
+    [[maybe_unused]] const int c4 = co0 + c0 + 4 * (lane & 3);
+    // dy of four channels at offset q where the ReLU output m passed
+    [[maybe_unused]] auto emit = [&](float* g, uint2 m, size_t q) {
+      const float2 m0 = unpack_bf16(m.x), m1 = unpack_bf16(m.y);
+      g[0] = m0.x > 0.f ? g[0] : 0.f;
+      g[1] = m0.y > 0.f ? g[1] : 0.f;
+      g[2] = m1.x > 0.f ? g[2] : 0.f;
+      g[3] = m1.y > 0.f ? g[3] : 0.f;
 #pragma unroll
-      for (int e = 0; e < 16; e++) bsum[e] = 0.f;
-    }
-    // dy of eight channels at offset q, sums from channel e0 on
-    auto emit = [&](float* g, uint4 mask, size_t q, int e0) {
-      float m[8];
-      unpack8(mask, m);
-#pragma unroll
-      for (int e = 0; e < 8; e++) {
-        g[e] = m[e] > 0.f ? g[e] : 0.f;
-        bsum[e0 + e] += g[e];
-      }
-      store8(a.dy32 + q, g);
-      *reinterpret_cast<uint4*>(a.dy16 + q) = pack8(g);
+      for (int e = 0; e < 4; e++) bsum[e] += g[e];
+      store4(a.dy32 + q, g);
+      *reinterpret_cast<uint2*>(a.dy16 + q) = make_uint2(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]));
     };
     TileRun r;
     for (int u = lo; ok && next_run(u, hi, a.H, r);) {
@@ -466,14 +482,21 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
           sk0 = __ldg(reinterpret_cast<const uint4*>(a.skip + o));
           sk1 = __ldg(reinterpret_cast<const uint4*>(a.skip + o) + 1);
         }
-        [[maybe_unused]] size_t oq = 0;       // kEpiDown: this lane's eight channels of the pixel pair
+        // the masks of the quad's four pixels (kEpiDown: of its two pixel pairs, on odd rows)
+        const int p0 = r.seg * kM + qw * 32 + (lane & ~3);
+        [[maybe_unused]] uint2 mk[4];
         if constexpr (kEpi == kEpiMask) {
-          sk0 = __ldg(reinterpret_cast<const uint4*>(a.mask + o));
-          sk1 = __ldg(reinterpret_cast<const uint4*>(a.mask + o) + 1);
+#pragma unroll
+          for (int k = 0; k < 4; k++)
+            mk[k] = __ldg(reinterpret_cast<const uint2*>(a.mask + ((size_t)y * a.W + min(p0 + k, a.W - 1)) * a.Cout + c4));
         }
         if constexpr (kEpi == kEpiDown) {
-          oq = ((size_t)(y >> 1) * (a.W >> 1) + (in ? px >> 1 : 0)) * a.Cout + co0 + c0 + ((lane & 1) ? 8 : 0);
-          if (y & 1) sk0 = __ldg(reinterpret_cast<const uint4*>(a.mask + oq));
+          if (y & 1) {
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+              mk[k] = __ldg(reinterpret_cast<const uint2*>(
+                  a.mask + ((size_t)(y >> 1) * (a.W >> 1) + min((p0 >> 1) + k, (a.W >> 1) - 1)) * a.Cout + c4));
+          }
         }
         if (!(ok = mbar_wait(&acc_full[b], (tc >> 1) & 1u, 64))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -491,66 +514,55 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
           const float val = __uint_as_float(v[e]) + bias_s[c0 + e];
           f[e] = a.relu ? fmaxf(val, 0.f) : val;
         }
-        if constexpr (kEpi == kEpiPlain) {
-          if (in) {
-            store8(a.y32 + o, f);
-            store8(a.y32 + o + 8, f + 8);
+        if constexpr (kEpi == kEpiPlain || epi_gradient(kEpi)) {
+          float t[4][4];
+#pragma unroll
+          for (int e = 0; e < 16; e++) t[e >> 2][e & 3] = f[e];
+          quad_transpose(t, lane);
+          if constexpr (kEpi == kEpiPlain || kEpi == kEpiMask) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+              if (p0 + k >= a.W) continue;
+              const size_t q = ((size_t)y * a.W + p0 + k) * a.Cout + c4;
+              store4((kEpi == kEpiPlain ? a.y32 : a.raw32) + q, t[k]);
+              if constexpr (kEpi == kEpiMask) emit(t[k], mk[k], q);
+            }
+          } else if constexpr (kEpi == kEpiDown) {
+            if (y & 1) {
+#pragma unroll
+              for (int k = 0; k < 2; k++) {
+                if (p0 + 2 * k >= a.W) continue;      // W is even
+                float g[4];
+#pragma unroll
+                for (int e = 0; e < 4; e++)
+                  g[e] = ((prow[2 * k][e] + prow[2 * k + 1][e]) + t[2 * k][e]) + t[2 * k + 1][e];
+                const size_t q = ((size_t)(y >> 1) * (a.W >> 1) + (p0 >> 1) + k) * a.Cout + c4;
+                if (a.raw32) store4(a.raw32 + q, g);
+                emit(g, mk[k], q);
+              }
+            } else {
+#pragma unroll
+              for (int e = 0; e < 16; e++) prow[e >> 2][e & 3] = t[e >> 2][e & 3];
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+              if (p0 + k >= a.W) continue;
+#pragma unroll
+              for (int d = 0; d < 4; d++) {
+                const size_t q = ((size_t)(2 * y + (d >> 1)) * (2 * a.W) + 2 * (p0 + k) + (d & 1)) * a.Cout + c4;
+                const uint2 m = __ldg(reinterpret_cast<const uint2*>(a.mask + q));
+                const float4 u = __ldg(reinterpret_cast<const float4*>(a.add32 + q));
+                float g[4] = {u.x + 0.25f * t[k][0], u.y + 0.25f * t[k][1], u.z + 0.25f * t[k][2], u.w + 0.25f * t[k][3]};
+                emit(g, m, q);
+              }
+            }
           }
           continue;
         }
         // Lanes past the row's end compute on their TMEM rows and take part in
         // the exchanges; they store only their partner's pixel.
         const bool odd = (lane & 1) != 0;
-        if constexpr (kEpi == kEpiMask) {
-          if (in) {
-            store8(a.raw32 + o, f);
-            store8(a.raw32 + o + 8, f + 8);
-            emit(f, sk0, o, 0);
-            emit(f + 8, sk1, o + 8, 8);
-          }
-          continue;
-        }
-        if constexpr (kEpi == kEpiDown) {
-          // the even lane sums channels 0-7 of the pair, the odd lane 8-15
-          if (y & 1) {
-            float g[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-              const float r0 = __shfl_xor_sync(0xffffffffu, odd ? prow[e] : prow[8 + e], 1);
-              const float r1 = __shfl_xor_sync(0xffffffffu, odd ? f[e] : f[8 + e], 1);
-              const float x00 = odd ? r0 : prow[e], x01 = odd ? prow[8 + e] : r0;
-              const float x10 = odd ? r1 : f[e], x11 = odd ? f[8 + e] : r1;
-              g[e] = ((x00 + x01) + x10) + x11;
-            }
-            if (in) {
-              if (a.raw32) store8(a.raw32 + oq, g);
-              emit(g, sk0, oq, 0);
-            }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 16; e++) prow[e] = f[e];
-          }
-          continue;
-        }
-        if constexpr (kEpi == kEpiSpread) {
-          if (in) {
-#pragma unroll
-            for (int d = 0; d < 4; d++) {
-              const size_t q = ((size_t)(2 * y + (d >> 1)) * (2 * a.W) + 2 * px + (d & 1)) * a.Cout + co0 + c0;
-#pragma unroll
-              for (int h = 0; h < 2; h++) {
-                const uint4 m = __ldg(reinterpret_cast<const uint4*>(a.mask + q) + h);
-                const float4 u0 = __ldg(reinterpret_cast<const float4*>(a.add32 + q) + 2 * h);
-                const float4 u1 = __ldg(reinterpret_cast<const float4*>(a.add32 + q) + 2 * h + 1);
-                float g[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-                for (int e = 0; e < 8; e++) g[e] = g[e] + 0.25f * f[8 * h + e];
-                emit(g, m, q + 8 * h, 8 * h);
-              }
-            }
-          }
-          continue;
-        }
         uint4 h0 = pack8(f), h1 = pack8(f + 8);
         if constexpr (kEpi == kEpiPool) {
           // W and H are even: both pixels and both rows of a pair are inside.
@@ -619,17 +631,11 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
       }
     }
     if constexpr (epi_gradient(kEpi)) {
-      // kEpiDown: even lanes hold channels 0-7, odd lanes 8-15
-      constexpr int kCh = kEpi == kEpiDown ? 8 : 16;
 #pragma unroll
-      for (int e = 0; e < kCh; e++)
+      for (int e = 0; e < 4; e++)
 #pragma unroll
-        for (int m = 16; m >= (kEpi == kEpiDown ? 2 : 1); m >>= 1) bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], m);
-      float* d = a.bpart + (size_t)(4 * blockIdx.x + qw) * a.Cout + co0 + c0;
-      if (lane < 16 / kCh) {
-#pragma unroll
-        for (int e = 0; e < kCh; e++) d[kCh * lane + e] = bsum[e];
-      }
+        for (int m = 16; m >= 4; m >>= 1) bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], m);
+      if (lane < 4) store4(a.bpart + (size_t)(4 * blockIdx.x + qw) * a.Cout + c4, bsum);
     }
   }
   if (!ok && (lane == 0)) atomicOr(a.status, 1u);

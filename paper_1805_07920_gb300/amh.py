@@ -151,8 +151,9 @@ def fuse(cams, depths, normals, f_eps=0.3, f_ang_deg=30.0, f_con=2):
     arr = make_cameras(cams)
     d = [x.contiguous() for x in depths]
     n = [x.contiguous() for x in normals]
-    pts = [torch.zeros(x.shape[0], x.shape[1], 6, dtype=torch.float32, device=x.device) for x in d]
-    cnt = [torch.zeros(x.shape[0], x.shape[1], dtype=torch.uint8, device=x.device) for x in d]
+    # every element is written by the kernel
+    pts = [torch.empty(x.shape[0], x.shape[1], 6, dtype=torch.float32, device=x.device) for x in d]
+    cnt = [torch.empty(x.shape[0], x.shape[1], dtype=torch.uint8, device=x.device) for x in d]
     keep = []
 
     def P(ts):

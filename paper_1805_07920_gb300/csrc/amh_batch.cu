@@ -125,10 +125,8 @@ __global__ void __launch_bounds__(kBThreads, kBBlocksPerSM) batch_phase_kernel(c
     const int ty = local / ra.tiles_x, tx = local % ra.tiles_x;
     const int y = ty * T::rows + T::row(threadIdx.x);
     const int x = tx * TW + 2 * T::col(threadIdx.x) + ((y + b.color) & 1);
-    if (x < ra.W && y < ra.H) {
-      PixelArrays sm;
-      update_pixel<kHalf, kMode>(ra, sm, x, y, &npairs, ws.q + threadIdx.x);
-    }
+    PixelArrays sm;
+    update_pixel<kHalf, kMode>(ra, sm, x, y, &npairs, ws.q + threadIdx.x, ws.slots[threadIdx.x >> 5], x < ra.W && y < ra.H);
   }
   const int tot = __reduce_add_sync(0xffffffffu, npairs);
   if ((threadIdx.x & 31) == 0 && tot)

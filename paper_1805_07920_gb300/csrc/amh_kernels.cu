@@ -51,11 +51,11 @@ __global__ void __launch_bounds__(kThreads, (kMode & kStage) ? kStagedBlocksPerS
     const int x = blockIdx.x * kTile + 2 * (4 * (q & 1) + (lane & 3)) + ((y + a.color) & 1);
     // the whole block takes part in the staged sweep, pixels outside the image too
     __shared__ StageShared ss;
-    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, &ss, x < a.W && y < a.H);
+    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H, &ss);
   } else {
     const int y = blockIdx.y * kTile + (tid >> 3);
     const int x = blockIdx.x * kTile + 2 * (tid & 7) + ((y + a.color) & 1);
-    if (x < a.W && y < a.H) update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid);
+    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H);
   }
   count_pairs(a, npairs);
 }

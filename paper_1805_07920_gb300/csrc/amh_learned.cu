@@ -119,27 +119,28 @@ __global__ void __launch_bounds__(256) l1_loss_kernel(const float* __restrict__ 
                                                       float* loss, int np) {
   const float inv_n = 1.f / (float)max(1u, *count);
   float s = 0.f, gs[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
-    const float4 o = reinterpret_cast<const float4*>(out)[(size_t)p * 4];
-    const float4 t = reinterpret_cast<const float4*>(target)[p];
-    const bool on = mask[p] != 0;
-    const float d[4] = {o.x - t.x, o.y - t.y, o.z - t.z, o.w - t.w};
-    float g[4];
+  // four threads per pixel, each a quarter of its channels: the first has the
+  // used ones, the others store zeros
+  const int q = threadIdx.x & 3;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 4 * (int64_t)np; i += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(i >> 2);
+    float g[4] = {0.f, 0.f, 0.f, 0.f};
+    if (q == 0) {
+      const float4 o = reinterpret_cast<const float4*>(out)[(size_t)p * 4];
+      const float4 t = reinterpret_cast<const float4*>(target)[p];
+      const bool on = mask[p] != 0;
+      const float d[4] = {o.x - t.x, o.y - t.y, o.z - t.z, o.w - t.w};
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      g[c] = 0.f;
-      if (on) {
-        s += fabsf(d[c]);
-        g[c] = (d[c] > 0.f ? 1.f : (d[c] < 0.f ? -1.f : 0.f)) * inv_n;
+      for (int c = 0; c < 4; c++) {
+        if (on) {
+          s += fabsf(d[c]);
+          g[c] = (d[c] > 0.f ? 1.f : (d[c] < 0.f ? -1.f : 0.f)) * inv_n;
+        }
+        gs[c] += g[c];
       }
-      gs[c] += g[c];
     }
-    float4* dp = reinterpret_cast<float4*>(dout) + (size_t)p * 4;
-    dp[0] = make_float4(g[0], g[1], g[2], g[3]);
-    dp[1] = dp[2] = dp[3] = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint4* dh = reinterpret_cast<uint4*>(dout16) + (size_t)p * 2;
-    dh[0] = make_uint4(tc::pack_bf16(g[0], g[1]), tc::pack_bf16(g[2], g[3]), 0u, 0u);
-    dh[1] = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<float4*>(dout)[i] = make_float4(g[0], g[1], g[2], g[3]);
+    reinterpret_cast<uint2*>(dout16)[i] = make_uint2(tc::pack_bf16(g[0], g[1]), tc::pack_bf16(g[2], g[3]));
   }
   __shared__ float red[8][5];
 #pragma unroll
@@ -215,7 +216,9 @@ __global__ void features_kernel(const void* ref, int ref_half, const float4* pla
     const float4 pl = plane[qs];
     const float f[6] = {I / 255.f - 0.5f, (logf(fmaxf(pl.w, 1e-6f)) - lmid) * lscale, pl.x, pl.y, pl.z,
                         cost[qs] * 0.5f};
-    for (int c = 0; c < 16; c++) x0[(size_t)p * 16 + c] = __float2bfloat16(c < 6 ? f[c] : 0.f);
+    uint4* xr = reinterpret_cast<uint4*>(x0) + (size_t)p * 2;
+    xr[0] = make_uint4(tc::pack_bf16(f[0], f[1]), tc::pack_bf16(f[2], f[3]), tc::pack_bf16(f[4], f[5]), 0u);
+    xr[1] = make_uint4(0u, 0u, 0u, 0u);
     pin[p] = pl;
   }
 }
@@ -310,6 +313,12 @@ struct ConvOp {
   int threads;
   size_t smem;
 };
+struct WgradOp {
+  CUtensorMap mdy, mx;
+  tc::WgradTcArgs a;
+  dim3 grid;
+  size_t smem;
+};
 struct amh_net {
   int w2 = 0, h2 = 0;                     // network input size (half resolution)
   cudaStream_t stream = nullptr;
@@ -344,6 +353,7 @@ struct amh_net {
   float *gE1 = nullptr, *gE2 = nullptr, *gE3 = nullptr;
   float* scratch = nullptr;               // 64 floats per pixel: host examples, tensors read back
   ConvOp fwd[kLayers], dgr[kLayers];      // forward; data gradients (layer 0 has none)
+  WgradOp wgr[kLayers];
   float* loss = nullptr;
   unsigned int* count = nullptr;          // sum of the mask
   unsigned int* status = nullptr;         // bit 0: a convolution's barrier wait gave up
@@ -426,7 +436,7 @@ const void* conv_kernel(int epi) {
     default: return reinterpret_cast<const void*>(tc::conv3x3_tc_kernel<tc::kEpiPlain>);
   }
 }
-// Launch of a convolution.  overlap: its set-up (barriers, tensor memory,
+// Launch of a tensor-core kernel.  overlap: its set-up (barriers, tensor memory,
 // weights) may start while the kernel before it on the stream is still running;
 // the kernel itself waits for that one before it reads or writes anything else.
 // The weights are read during set-up, so they must be complete one ordinary
@@ -501,6 +511,7 @@ int conv(amh_net* n, ConvOp& op, bool overlap) {
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "conv launch: %s", cudaGetErrorString(e));
   return AMH_OK;
 }
+int plan_wgrad(amh_net* n, WgradOp& op, int L, const __nv_bfloat16* x, int H, int W);
 // every convolution of the forward and backward pass
 int plan_network(amh_net* n) {
   const int W0 = n->w2, H0 = n->h2, W1 = W0 / 2, H1 = H0 / 2, W2 = W1 / 2, H2 = H1 / 2, W3 = W2 / 2, H3 = H2 / 2;
@@ -559,41 +570,39 @@ int plan_network(amh_net* n) {
     n->brows[d[L].to] = 4 * (int)n->dgr[L].grid.x;
     if (!rc && n->brows[d[L].to] > kBiasRows) rc = nfail(n, AMH_EINVAL, "conv: more partial sums than rows");
   }
+  for (int L = 0; L < kLayers && !rc; L++) rc = plan_wgrad(n, n->wgr[L], L, f[L].x, f[L].H, f[L].W);
   return rc;
 }
 // weight gradient of layer L from its input x and its output gradient (BF16
 // dy16): the tensor-core kernel reads both pixel-major and sums a band of rows
 // per CTA (all nine taps when Cout <= 32, else the three of one vertical tap)
 // into gw
-int wgrad(amh_net* n, int L, const __nv_bfloat16* x, int H, int W) {
+int plan_wgrad(amh_net* n, WgradOp& op, int L, const __nv_bfloat16* x, int H, int W) {
   const int Cin = kNet[L].cin, Cout = kNet[L].cout;
-  const __nv_bfloat16* dy16 = n->dy16[L];
   const int stacked = Cout <= 32 ? 1 : 0, cba = stacked ? Cout : 64, cbb = tc::wgrad_xbox(Cin);
-  CUtensorMap mdy, mx;
-  if (!bf16_map(&mdy, dy16, Cout, W, H, cba, 64, 1, 0, block_swizzle(cba)) ||
-      !bf16_map(&mx, x, Cin, W, H, cbb, 66, 1, 0, block_swizzle(cbb)))
+  if (!bf16_map(&op.mdy, n->dy16[L], Cout, W, H, cba, 64, 1, 0, block_swizzle(cba)) ||
+      !bf16_map(&op.mx, x, Cin, W, H, cbb, 66, 1, 0, block_swizzle(cbb)))
     return nfail(n, AMH_ECUDA, "wgrad: tensor map encoding failed");
   const int S = tc::wgrad_stages(Cin);
-  const size_t smem = (size_t)S * tc::wgrad_stage_bytes(Cin) + tc::kWgSlack;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  static std::once_flag once[64];
-  static cudaError_t attr_err[64] = {};
-  std::call_once(once[dev & 63], [dev] {
-    attr_err[dev & 63] = cudaFuncSetAttribute(tc::wgrad3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(tc::kWgSmemCap + tc::kWgSlack));
-  });
-  if (attr_err[dev & 63] != cudaSuccess)
-    return nfail(n, AMH_ECUDA, "wgrad: shared-memory attribute: %s", cudaGetErrorString(attr_err[dev & 63]));
-  int n_sm = 0;
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  op.smem = (size_t)S * tc::wgrad_stage_bytes(Cin) + tc::kWgSlack;
+  int dev = 0, n_sm = 0;
+  cudaError_t e = cudaFuncSetAttribute(tc::wgrad3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(tc::kWgSmemCap + tc::kWgSlack));
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "wgrad: kernel attributes: %s", cudaGetErrorString(e));
   // one CTA per SM (the ring takes most of the shared memory), each an equal
   // share of the (row, 64-pixel chunk) steps
   const int gy = stacked ? 1 : 3, steps = H * ((W + 63) / 64);
   const int per_cta = (steps + std::max(1, n_sm / gy) - 1) / std::max(1, n_sm / gy);
-  const tc::WgradTcArgs a{n->gw[L], n->status, H, W, Cin, Cout, per_cta, stacked, S};
-  tc::wgrad3x3_tc_kernel<<<dim3((steps + per_cta - 1) / per_cta, gy), tc::kThreads, smem, n->stream>>>(mdy, mx, a);
-  const cudaError_t e = cudaGetLastError();
+  op.a = tc::WgradTcArgs{n->gw[L], n->status, H, W, Cin, Cout, per_cta, stacked, S};
+  op.grid = dim3((steps + per_cta - 1) / per_cta, gy);
+  return AMH_OK;
+}
+int wgrad(amh_net* n, WgradOp& op) {
+  void* args[] = {&op.mdy, &op.mx, &op.a};
+  const cudaError_t e = launch_conv(reinterpret_cast<const void*>(tc::wgrad3x3_tc_kernel), op.grid, tc::kThreads, op.smem,
+                                    n->stream, true, args);
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "wgrad launch: %s", cudaGetErrorString(e));
   return AMH_OK;
 }
@@ -762,7 +771,6 @@ AMH_API int amh_net_features(amh_net* n, amh_ctx* c) {
   if ((c->W + 1) / 2 > n->w2 || (c->H + 1) / 2 > n->h2) return nfail(n, AMH_EINVAL, "context larger than the network");
   const float lmid = 0.5f * (std::log(c->p.depth_min) + std::log(c->p.depth_max));
   const float lscale = 2.f / std::max(1e-6f, std::log(c->p.depth_max / c->p.depth_min));
-  NTRY(n, cudaMemsetAsync(n->x0, 0, (size_t)n->w2 * n->h2 * 16 * 2, n->stream));
   features_kernel<<<blocks_for((size_t)n->w2 * n->h2), 256, 0, n->stream>>>(
       c->d_ref, c->args.img_half, c->d_plane, c->d_cost, c->W, c->H, n->w2, n->h2, lmid, lscale, n->x0, n->pin);
   NTRY(n, cudaGetLastError());
@@ -808,13 +816,12 @@ AMH_API int amh_net_backward(amh_net* n, float* loss_out) {
   // gradients, loss and the mask's sum
   NTRY(n, cudaMemsetAsync(n->gw[0], 0, (n->n_params + 2) * sizeof(float), s));
   mask_count_kernel<<<(int)std::min<size_t>((P0 / 16 + 255) / 256, 152), 256, 0, s>>>(n->mask, (int)P0, n->count);
-  const int lb = (int)std::min<size_t>((P0 + 255) / 256, kBiasRows);
+  const int lb = (int)std::min<size_t>((P0 * 4 + 255) / 256, kBiasRows);
   l1_loss_kernel<<<lb, 256, 0, s>>>(n->out, n->target, n->mask, n->count, n->dy[7], n->dy16[7], n->bpart[7], n->loss, (int)P0);
   n->brows[7] = lb;
-  const __nv_bfloat16* x[kLayers] = {n->x0, n->in_e2, n->in_e3, n->in_e4, n->in_d3, n->in_d2, n->in_d1, n->d1};
   int rc = AMH_OK;
   for (int L = kLayers - 1; L >= 0 && !rc; L--) {
-    rc = wgrad(n, L, x[L], n->fwd[L].a.H, n->fwd[L].a.W);
+    rc = wgrad(n, n->wgr[L]);
     if (!rc && L > 0) rc = conv(n, n->dgr[L], true);
   }
   BiasArgs ba;

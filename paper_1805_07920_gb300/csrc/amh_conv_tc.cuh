@@ -270,6 +270,7 @@ struct ConvTcArgs {
   float* bpart;               // sums of dy per CTA and lane quarter: row 4 blockIdx.x + quarter, Cout channels
   unsigned int* status;       // bit 0: a barrier wait gave up
   int H, W, Cin, Cout, relu;
+  int row0, rows;             // output rows row0 .. row0 + rows - 1
   int Nb;                     // output channels per CTA (a multiple of 16 dividing Cout, at most kConvMaxNb)
   int S;                      // slab stages (3 .. kMaxStages)
 };
@@ -327,8 +328,8 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int w_prod = 4 * (Nb / 16), w_mma = w_prod + 1;
   const int co0 = blockIdx.y * Nb;
-  const int nseg = (a.W + kM - 1) / kM, ntiles = a.H * nseg;
-  // with row pairs (H even) every range starts and ends at an even row
+  const int nseg = (a.W + kM - 1) / kM, ntiles = a.rows * nseg;
+  // with row pairs (rows even, row0 = 0) every range starts and ends at an even row
   constexpr int kUnit = epi_row_pairs(kEpi) ? 2 : 1;
   const int lo = kUnit * (int)((int64_t)(ntiles / kUnit) * blockIdx.x / gridDim.x);
   const int hi = kUnit * (int)((int64_t)(ntiles / kUnit) * (blockIdx.x + 1) / gridDim.x);
@@ -371,14 +372,14 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
       pdl_launch();
       RingPos q{0u, 0u};
       TileRun r;
-      for (int u = lo; ok && next_run(u, hi, a.H, r);) {
+      for (int u = lo; ok && next_run(u, hi, a.rows, r);) {
         const int x0 = r.seg * kM;
         for (int k = 0; k < r.len + 2 && ok; k++, q = q.next((uint32_t)S)) {
           if (!(ok = mbar_wait(&empty[q.slot], q.phase ^ 1u))) break;
           mbar_expect_tx(&full[q.slot], (uint32_t)kHalo * 2u * (uint32_t)a.Cin);
           uint8_t* dst = slabs + (size_t)q.slot * slab_bytes;
           for (int bk = 0; bk < nblk; bk++)
-            tma_load_3d(dst + (size_t)bk * sblk, bk < nmain ? &tx_main : &tx_tail, 64 * bk, x0 - 1, r.y0 - 1 + k,
+            tma_load_3d(dst + (size_t)bk * sblk, bk < nmain ? &tx_main : &tx_tail, 64 * bk, x0 - 1, a.row0 + r.y0 - 1 + k,
                         &full[q.slot]);
         }
       }
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
       uint32_t tc = 0;
       RingPos q{0u, 0u};    // ring position of the next slab
       TileRun r;
-      for (int u = lo; ok && next_run(u, hi, a.H, r);) {
+      for (int u = lo; ok && next_run(u, hi, a.rows, r);) {
         RingPos q0 = q, q1 = q.next((uint32_t)S);    // slabs i and i + 1 of the run
         for (int i = 0; i < r.len && ok; i++, tc++) {
           const uint32_t b = tc & 1u;
@@ -470,10 +471,10 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv3x3_tc_kernel(const __
       *reinterpret_cast<uint2*>(a.dy16 + q) = make_uint2(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]));
     };
     TileRun r;
-    for (int u = lo; ok && next_run(u, hi, a.H, r);) {
+    for (int u = lo; ok && next_run(u, hi, a.rows, r);) {
       for (int i = 0; i < r.len && ok; i++, tc++) {
         const uint32_t b = tc & 1u;
-        const int y = r.y0 + i, px = r.seg * kM + qw * 32 + lane;
+        const int y = a.row0 + r.y0 + i, px = r.seg * kM + qw * 32 + lane;
         const bool in = px < a.W;
         const size_t o = ((size_t)y * a.W + (in ? px : 0)) * a.Cout + co0 + c0;
         // this lane's skip values, fetched while the tile's MMAs run

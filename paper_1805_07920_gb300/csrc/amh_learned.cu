@@ -41,6 +41,7 @@ namespace amh {
 namespace {
 
 constexpr int kLayers = 8;
+constexpr int kMaxBands = 4;            // bands of rows of the last two layers (amh_net_forward with an output)
 struct LayerDef { int cin, cout, relu; };
 // e1 e2 e3 e4 d3 d2 d1 out
 constexpr LayerDef kNet[kLayers] = {{16, 32, 1}, {32, 64, 1}, {64, 96, 1}, {96, 128, 1},
@@ -354,6 +355,11 @@ struct amh_net {
   float* scratch = nullptr;               // 64 floats per pixel: host examples, tensors read back
   ConvOp fwd[kLayers], dgr[kLayers];      // forward; data gradients (layer 0 has none)
   WgradOp wgr[kLayers];
+  // the output's copy to the host, beside the layers that compute its later rows
+  cudaStream_t side = nullptr;
+  cudaEvent_t ready = nullptr, done = nullptr;
+  int n_bands = 0;
+  ConvOp band[2 * kMaxBands];             // the last two layers in bands of rows
   float* loss = nullptr;
   unsigned int* count = nullptr;          // sum of the mask
   unsigned int* status = nullptr;         // bit 0: a convolution's barrier wait gave up
@@ -389,6 +395,13 @@ cudaError_t nalloc(amh_net* n, T** p, size_t count) {
                    cudaGetErrorString(e_));                                                    \
   } while (0)
 
+void free_net(amh_net* n) {
+  if (n->side) cudaStreamDestroy(n->side);
+  if (n->ready) cudaEventDestroy(n->ready);
+  if (n->done) cudaEventDestroy(n->done);
+  for (void* p : n->allocs) cudaFree(p);
+  delete n;
+}
 // the driver's tensor-map encoder, looked up once through the runtime
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -478,6 +491,7 @@ int plan_conv(amh_net* n, ConvOp& op, const __nv_bfloat16* x, const __nv_bfloat1
   if (Cin < 64) op.mx[0] = op.mx[1], op.mw[0] = op.mw[1];
   if (!tail) op.mx[1] = op.mx[0], op.mw[1] = op.mw[0];
   a.status = n->status;
+  if (!a.rows) a.rows = H;                  // all rows
   a.H = H;
   a.W = W;
   a.Cin = Cin;
@@ -501,7 +515,7 @@ int plan_conv(amh_net* n, ConvOp& op, const __nv_bfloat16* x, const __nv_bfloat1
   // the register file; at most one per tile (or pair of tiles)
   const int by_regs = 65536 / (((fa.numRegs + 7) & ~7) * op.threads);
   const int cps = std::max(1, std::min(p.ctas_per_sm, by_regs));
-  const int nblk = Cout / p.Nb, ntiles = H * ((W + tc::kM - 1) / tc::kM) / (tc::epi_row_pairs(epi) ? 2 : 1);
+  const int nblk = Cout / p.Nb, ntiles = a.rows * ((W + tc::kM - 1) / tc::kM) / (tc::epi_row_pairs(epi) ? 2 : 1);
   op.grid = dim3(std::max(1, std::min(ntiles, n_sm * cps / nblk)), nblk);
   return AMH_OK;
 }
@@ -570,6 +584,19 @@ int plan_network(amh_net* n) {
     n->brows[d[L].to] = 4 * (int)n->dgr[L].grid.x;
     if (!rc && n->brows[d[L].to] > kBiasRows) rc = nfail(n, AMH_EINVAL, "conv: more partial sums than rows");
   }
+  // band b of the last layer: rows [H0 b / n, H0 (b + 1) / n); of the layer before
+  // it: the rows those need that no earlier band computed (one row ahead)
+  n->n_bands = std::max(1, std::min(kMaxBands, H0 / 32));
+  for (int b = 0; b < n->n_bands && !rc; b++) {
+    const int r0 = H0 * b / n->n_bands, r1 = H0 * (b + 1) / n->n_bands;
+    for (int l = 0; l < 2 && !rc; l++) {
+      const int L = kLayers - 2 + l;
+      tc::ConvTcArgs a = n->fwd[L].a;
+      a.row0 = l ? r0 : b ? r0 + 1 : 0;
+      a.rows = (l || r1 == H0 ? r1 : r1 + 1) - a.row0;
+      rc = plan_conv(n, n->band[2 * b + l], f[L].x, n->w16[L], H0, W0, kNet[L].cin, kNet[L].cout, f[L].epi, a);
+    }
+  }
   for (int L = 0; L < kLayers && !rc; L++) rc = plan_wgrad(n, n->wgr[L], L, f[L].x, f[L].H, f[L].W);
   return rc;
 }
@@ -606,6 +633,28 @@ int wgrad(amh_net* n, WgradOp& op) {
   if (e != cudaSuccess) return nfail(n, AMH_ECUDA, "wgrad launch: %s", cudaGetErrorString(e));
   return AMH_OK;
 }
+// the last two layers in bands, each band's output on its way to the host's
+// pinned memory as soon as it is there; the main stream waits for the copies.
+// After a failure no copy is left in flight.
+int forward_bands(amh_net* n, float* out_host) {
+  cudaError_t e = cudaSuccess;
+  int rc = AMH_OK;
+  for (int b = 0; b < n->n_bands && !rc && e == cudaSuccess; b++) {
+    rc = conv(n, n->band[2 * b], true);
+    if (!rc) rc = conv(n, n->band[2 * b + 1], true);
+    if (rc) break;
+    const tc::ConvTcArgs& a = n->band[2 * b + 1].a;
+    const size_t first = (size_t)a.row0 * a.W * 16, count = (size_t)a.rows * a.W * 16;
+    e = cudaEventRecord(n->ready, n->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(n->side, n->ready, 0);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(out_host + first, n->out + first, count * 4, cudaMemcpyDeviceToHost, n->side);
+  }
+  if (!rc && e == cudaSuccess) e = cudaEventRecord(n->done, n->side);
+  if (!rc && e == cudaSuccess) e = cudaStreamWaitEvent(n->stream, n->done, 0);
+  if (rc || e != cudaSuccess) cudaStreamSynchronize(n->side);
+  return rc ? rc : e == cudaSuccess ? AMH_OK : nfail(n, AMH_ECUDA, "output copy: %s", cudaGetErrorString(e));
+}
 }  // namespace
 
 extern "C" {
@@ -623,8 +672,7 @@ AMH_API int amh_net_create(amh_net** out, int32_t width2, int32_t height2, uint6
   n->stream = (cudaStream_t)stream;
   auto bail = [&](int code) {
     g_net_err = n->err;
-    for (void* p : n->allocs) cudaFree(p);
-    delete n;
+    free_net(n);
     return code;
   };
 #define NA(p, c)                                                  \
@@ -685,6 +733,13 @@ AMH_API int amh_net_create(amh_net** out, int32_t width2, int32_t height2, uint6
   NA(n->gE1, P0 * 32); NA(n->gE2, P1 * 64); NA(n->gE3, P2 * 96);
   NA(n->out, P0 * 16); NA(n->target, P0 * 4); NA(n->mask, P0); NA(n->pin, P0); NA(n->prop, P0);
 #undef NA
+  cudaError_t se = cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking);
+  if (se == cudaSuccess) se = cudaEventCreateWithFlags(&n->ready, cudaEventDisableTiming);
+  if (se == cudaSuccess) se = cudaEventCreateWithFlags(&n->done, cudaEventDisableTiming);
+  if (se != cudaSuccess) {
+    nfail(n, AMH_ECUDA, "side stream: %s", cudaGetErrorString(se));
+    return bail(AMH_ECUDA);
+  }
   if (const int rc = plan_network(n)) return bail(rc);
   for (int L = 0; L < kLayers; L++) {
     const size_t nw = (size_t)9 * kNet[L].cin * kNet[L].cout;
@@ -798,7 +853,25 @@ AMH_API int amh_net_forward(amh_net* n, float* out_host) {
   if (!n) return AMH_EINVAL;
   const cudaStream_t s = n->stream;
   int rc = AMH_OK;
-  for (int L = 0; L < kLayers && !rc; L++) rc = conv(n, n->fwd[L], L > 0);
+  // An output to pinned memory is copied in bands of rows while the next band of
+  // the last two layers runs (the copy of 800 x 528 takes 142 us on the link,
+  // the two layers 55; with 1, 2, 3, 4, 6 bands 312, 292, 286, 284, 286 us).  A
+  // copy to pageable memory holds the host until it is done and goes last.
+  bool bands = false;
+  if (out_host) {
+    cudaPointerAttributes at;
+    const cudaError_t e = cudaPointerGetAttributes(&at, out_host);
+    if (e != cudaSuccess) cudaGetLastError();
+    bands = e == cudaSuccess && at.type == cudaMemoryTypeHost;
+  }
+  for (int L = 0; L < (bands ? kLayers - 2 : kLayers) && !rc; L++) rc = conv(n, n->fwd[L], L > 0);
+  if (bands) {
+    if (!rc) rc = forward_bands(n, out_host);
+    if (rc) return rc;
+    NTRY(n, cudaGetLastError());
+    NTRY(n, cudaStreamSynchronize(s));
+    return AMH_OK;
+  }
   if (rc) return rc;
   NTRY(n, cudaGetLastError());
   if (out_host) {
@@ -955,8 +1028,8 @@ AMH_API const char* amh_net_last_error(const amh_net* n) { return n ? n->err.c_s
 AMH_API void amh_net_destroy(amh_net* n) {
   if (!n) return;
   cudaStreamSynchronize(n->stream);
-  for (void* p : n->allocs) cudaFree(p);
-  delete n;
+  cudaStreamSynchronize(n->side);
+  free_net(n);
 }
 
 }  // extern "C"

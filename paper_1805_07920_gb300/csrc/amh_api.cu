@@ -21,18 +21,6 @@
 
 using namespace amh;
 
-namespace amh {
-// depth / normal split of the plane array into row-major maps
-__global__ void split_maps_kernel(const float4* __restrict__ plane, int W, int H, float* depth, float* normal3) {
-  const size_t n = (size_t)W * H;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 p = plane[state_index((int)(i % W), (int)(i / W), W)];
-    if (depth) depth[i] = p.w;
-    if (normal3) { normal3[3 * i] = p.x; normal3[3 * i + 1] = p.y; normal3[3 * i + 2] = p.z; }
-  }
-}
-}  // namespace amh
-
 // ===========================================================================
 // host side
 // ===========================================================================
@@ -490,30 +478,28 @@ AMH_API int amh_read_maps(amh_ctx* c, float* depth, float* normal3, float* cost,
                           int32_t mem) {
   if (!c) return AMH_EINVAL;
   if (mem != AMH_MEM_HOST && mem != AMH_MEM_DEVICE) return fail(c, AMH_EINVAL, "bad memory kind");
+  if (mem == AMH_MEM_DEVICE) {
+    CUDA_TRY(c, export_maps(c->d_plane, c->d_cost, c->d_wmask, c->W, c->H, depth, normal3, cost, selected, c->stream));
+    return AMH_OK;
+  }
   const size_t np = (size_t)c->W * c->H;
   if (depth || normal3) {
-    if (mem == AMH_MEM_DEVICE) {
-      split_maps_kernel<<<1024, 256, 0, c->stream>>>(c->d_plane, c->W, c->H, depth, normal3);
-      int rc = launch_check(c, "split_maps");
-      if (rc) return rc;
-    } else {
-      float* dd = nullptr;
-      float* dn = nullptr;
-      if (depth) CUDA_TRY(c, cudaMallocAsync(&dd, np * sizeof(float), c->stream));
-      if (normal3) CUDA_TRY(c, cudaMallocAsync(&dn, np * 3 * sizeof(float), c->stream));
-      split_maps_kernel<<<1024, 256, 0, c->stream>>>(c->d_plane, c->W, c->H, dd, dn);
-      int rc = launch_check(c, "split_maps");
-      if (!rc && depth) CUDA_TRY(c, cudaMemcpyAsync(depth, dd, np * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-      if (!rc && normal3)
-        CUDA_TRY(c, cudaMemcpyAsync(normal3, dn, np * 3 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-      if (dd) cudaFreeAsync(dd, c->stream);
-      if (dn) cudaFreeAsync(dn, c->stream);
-      if (rc) return rc;
-    }
+    float* dd = nullptr;
+    float* dn = nullptr;
+    if (depth) CUDA_TRY(c, cudaMallocAsync(&dd, np * sizeof(float), c->stream));
+    if (normal3) CUDA_TRY(c, cudaMallocAsync(&dn, np * 3 * sizeof(float), c->stream));
+    const cudaError_t e = export_maps(c->d_plane, nullptr, nullptr, c->W, c->H, dd, dn, nullptr, nullptr, c->stream);
+    int rc = e == cudaSuccess ? AMH_OK : fail(c, AMH_ECUDA, "read_maps launch: %s", cudaGetErrorString(e));
+    if (!rc && depth) CUDA_TRY(c, cudaMemcpyAsync(depth, dd, np * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    if (!rc && normal3)
+      CUDA_TRY(c, cudaMemcpyAsync(normal3, dn, np * 3 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    if (dd) cudaFreeAsync(dd, c->stream);
+    if (dn) cudaFreeAsync(dn, c->stream);
+    if (rc) return rc;
   }
-  if (cost) CUDA_TRY(c, export_state_field(c->d_cost, cost, c->W, c->H, 4, mem == AMH_MEM_HOST, c->stream));
-  if (selected) CUDA_TRY(c, export_state_field(c->d_wmask, selected, c->W, c->H, 4, mem == AMH_MEM_HOST, c->stream));
-  if (mem == AMH_MEM_HOST) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  if (cost) CUDA_TRY(c, export_state_field(c->d_cost, cost, c->W, c->H, 4, true, c->stream));
+  if (selected) CUDA_TRY(c, export_state_field(c->d_wmask, selected, c->W, c->H, 4, true, c->stream));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return AMH_OK;
 }
 

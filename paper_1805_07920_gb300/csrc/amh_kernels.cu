@@ -157,8 +157,19 @@ int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
   allow_dynamic(phase_team_kernel<kHalf, kTex, T>, once);
   const dim3 grid((a.W + 15) / 16, (a.H + 3) / 4);
-  phase_team_kernel<kHalf, kTex, T><<<grid, 32 * T, team_floats(a.N) * sizeof(float), s>>>(a);
-  return (int)cudaGetLastError();
+  // Small phases are short (10 - 20 us): the next one's blocks start loading their
+  // windows while this one's last blocks run.
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(32 * T);
+  cfg.dynamicSmemBytes = team_floats(a.N) * sizeof(float);
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return (int)cudaLaunchKernelEx(&cfg, phase_team_kernel<kHalf, kTex, T>, a);
 }
 
 template <bool kHalf, bool kTex>
@@ -224,23 +235,24 @@ int launch_phase(const PhaseArgs& a, cudaStream_t s) {
 namespace {
 // conversion between the state layout and row-major maps
 template <class T>
-__global__ void state_to_rows_kernel(const T* __restrict__ st, T* __restrict__ rows, int W, int H) {
-  const size_t n = (size_t)W * H;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    rows[i] = st[state_index((int)(i % W), (int)(i / W), W)];
+__global__ void __launch_bounds__(256) state_to_rows_kernel(const T* __restrict__ st, T* __restrict__ rows, int W, int H) {
+  const int x = blockIdx.x * 256 + threadIdx.x;
+  if (x >= W) return;
+  for (int y = blockIdx.y; y < H; y += gridDim.y) rows[(size_t)y * W + x] = st[state_index(x, y, W)];
 }
 template <class T>
-__global__ void rows_to_state_kernel(const T* __restrict__ rows, T* __restrict__ st, int W, int H) {
-  const size_t n = (size_t)W * H;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    st[state_index((int)(i % W), (int)(i / W), W)] = rows[i];
+__global__ void __launch_bounds__(256) rows_to_state_kernel(const T* __restrict__ rows, T* __restrict__ st, int W, int H) {
+  const int x = blockIdx.x * 256 + threadIdx.x;
+  if (x >= W) return;
+  for (int y = blockIdx.y; y < H; y += gridDim.y) st[state_index(x, y, W)] = rows[(size_t)y * W + x];
 }
 template <class T>
 void launch_convert(const void* src, void* dst, int W, int H, bool to_rows, cudaStream_t s) {
+  const dim3 grid((W + 255) / 256, H < 65535 ? H : 65535);
   if (to_rows)
-    state_to_rows_kernel<T><<<1024, 256, 0, s>>>(static_cast<const T*>(src), static_cast<T*>(dst), W, H);
+    state_to_rows_kernel<T><<<grid, 256, 0, s>>>(static_cast<const T*>(src), static_cast<T*>(dst), W, H);
   else
-    rows_to_state_kernel<T><<<1024, 256, 0, s>>>(static_cast<const T*>(src), static_cast<T*>(dst), W, H);
+    rows_to_state_kernel<T><<<grid, 256, 0, s>>>(static_cast<const T*>(src), static_cast<T*>(dst), W, H);
 }
 cudaError_t convert(const void* src, void* dst, int W, int H, int elem, bool to_rows, cudaStream_t s) {
   switch (elem) {
@@ -252,6 +264,38 @@ cudaError_t convert(const void* src, void* dst, int W, int H, int elem, bool to_
   return cudaGetLastError();
 }
 }  // namespace
+
+namespace {
+// the maps of amh_read_maps in one launch, row-major; any of them may be null
+__global__ void __launch_bounds__(256) export_maps_kernel(const float4* __restrict__ plane, const float* __restrict__ cost,
+                                                          const uint32_t* __restrict__ wmask, int W, int H,
+                                                          float* __restrict__ depth, float* __restrict__ normal3,
+                                                          float* __restrict__ cost_out, uint32_t* __restrict__ sel_out) {
+  const int x = blockIdx.x * 256 + threadIdx.x;
+  if (x >= W) return;
+  for (int y = blockIdx.y; y < H; y += gridDim.y) {
+    const size_t i = (size_t)y * W + x, q = state_index(x, y, W);
+    if (depth || normal3) {
+      const float4 p = plane[q];
+      if (depth) depth[i] = p.w;
+      if (normal3) {
+        normal3[3 * i] = p.x;
+        normal3[3 * i + 1] = p.y;
+        normal3[3 * i + 2] = p.z;
+      }
+    }
+    if (cost_out) cost_out[i] = cost[q];
+    if (sel_out) sel_out[i] = wmask[q];
+  }
+}
+}  // namespace
+cudaError_t export_maps(const float4* plane, const float* cost, const uint32_t* wmask, int W, int H, float* depth,
+                        float* normal3, float* cost_out, uint32_t* sel_out, cudaStream_t s) {
+  if (!depth && !normal3 && !cost_out && !sel_out) return cudaSuccess;
+  const dim3 grid((W + 255) / 256, H < 65535 ? H : 65535);
+  export_maps_kernel<<<grid, 256, 0, s>>>(plane, cost, wmask, W, H, depth, normal3, cost_out, sel_out);
+  return cudaGetLastError();
+}
 
 cudaError_t export_state_field(const void* state, void* rows, int W, int H, int elem, bool host, cudaStream_t s) {
   if (!host) return convert(state, rows, W, H, elem, true, s);

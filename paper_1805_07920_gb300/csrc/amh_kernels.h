@@ -15,4 +15,8 @@ int launch_phase(const PhaseArgs& a, cudaStream_t s);
 // Return the first cudaError_t met.
 cudaError_t export_state_field(const void* state, void* rows, int W, int H, int elem, bool host, cudaStream_t s);
 cudaError_t import_state_field(const void* rows, void* state, int W, int H, int elem, bool host, cudaStream_t s);
+// The maps of amh_read_maps (depth, 3-component normal, cost, selected views)
+// row-major in device memory, in one launch; any may be null.
+cudaError_t export_maps(const float4* plane, const float* cost, const uint32_t* wmask, int W, int H, float* depth,
+                        float* normal3, float* cost_out, uint32_t* sel_out, cudaStream_t s);
 }  // namespace amh

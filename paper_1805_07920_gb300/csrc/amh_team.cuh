@@ -33,6 +33,14 @@ struct TeamShared {
 // 8 j + g), psi_mod and one cost per view of 32 pixels
 __host__ __device__ constexpr int team_floats(int N) { return kTeamPixels * 10 * N; }
 
+// The launch before this one on the stream has finished and its state is
+// visible (the window depends on the image only, so it is loaded before); the
+// next launch may be set up from here on.
+__device__ __forceinline__ void phase_before_done() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // One colour phase's update of the team's 32 pixels; lane l's pixel is (x, y),
 // w the warp's index in the team (warp-uniform).  The whole block calls it.
 template <bool kHalf, bool kTex, int T, class A>
@@ -70,7 +78,9 @@ __device__ __forceinline__ void update_team(const A& a, TeamShared<T>& sh, float
     sh.stat[at(0)] = rw.inv_sw;
     sh.stat[at(1)] = rw.sum_wr;
     sh.stat[at(2)] = rw.var_r;
+    phase_before_done();
   } else {
+    phase_before_done();
     const int srow = 2 * ((a.W + 1) >> 1), xodd = x & 1;
     const int qbase = y * srow + (((x + y) & 1) ? 0 : (srow >> 1)) + (x >> 1);
     for (int g = w - 1; g < kRegions; g += T - 1) {
@@ -88,7 +98,7 @@ __device__ __forceinline__ void update_team(const A& a, TeamShared<T>& sh, float
           if (qx < 0 || qy < 0 || qx >= a.W || qy >= a.H) continue;
           const int q = (int)checked_index(a, (size_t)(qbase + dy * srow + ((xodd + dx) >> 1)), state_size(a.W, a.H),
                                            kBadNeighbour);
-          const float cq = __ldg(&a.cost[q]);
+          const float cq = a.cost[q];         // not a read-only load: the launch before may still write when this one starts
           if (best < 0 || cq < bc) { best = (dx + 32) | (dy + 32) << 8; bc = cq; }
         }
       }

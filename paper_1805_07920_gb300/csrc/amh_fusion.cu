@@ -105,13 +105,18 @@ __global__ void __launch_bounds__(32 * kMedWarps) median4_kernel(const float* __
     cswap(c[3], c[4]);
     cswap(c[5], c[6]);
     // and columns l + 2, l + 3
-    float m8, m9;
+    float lo[8], hi[8];
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const float d = __shfl_down_sync(0xffffffffu, c[7 - k], 2);
-      const float lo = fminf(c[k], d), hi = fmaxf(c[k], d);
-      m8 = k ? fmaxf(m8, lo) : lo;
-      m9 = k ? fminf(m9, hi) : hi;
+      lo[k] = fminf(c[k], d);
+      hi[k] = fmaxf(c[k], d);
+    }
+    float m8 = lo[0], m9 = hi[0];
+#pragma unroll
+    for (int k = 1; k < 8; k++) {
+      m8 = fmaxf(m8, lo[k]);
+      m9 = fminf(m9, hi[k]);
     }
     if (mine && y0 + r < (unsigned)H)
       out[(size_t)(y0 + r) * W + x] = sort_all ? median16_sorted(in, (int)x, (int)(y0 + r), W, H) : 0.5f * m8 + 0.5f * m9;

@@ -114,7 +114,7 @@ __device__ __forceinline__ void update_team(const A& a, TeamShared<T>& sh, float
   }
   sh.bits[0][at(w)] = valid;
   const uint32_t S_prev = a.sel[pi];
-  const int vb = a.vbest[pi], v_prev = vb == 255 ? -1 : vb;
+  const int v_prev = a.vbest[pi];         // 255: none
   float4 best = a.plane[pi];
   __syncthreads();
   rw.inv_sw = sh.stat[at(0)];
@@ -140,22 +140,12 @@ __device__ __forceinline__ void update_team(const A& a, TeamShared<T>& sh, float
   const int k = a.k < N ? a.k : N;
   uint32_t S = 0;
   for (int j = w; j < N; j += T) {
-    int ng = 0, nb = 0;
-    float psi = 0.f;
+    ViewScore score;
 #pragma unroll
-    for (int i = 0; i < kRegions; i++) {
-      if (!(valid >> i & 1u)) continue;
-      const float m = M[at(8 * j + i)];
-      ng += m < a.tau;
-      nb += m > a.tau_up;
-      psi += expf(-m * m * a.inv2beta2);          // Eq. (3)
-    }
-    float pm = 0.f;
-    if (ng > a.n1 && nb < a.n2) {                  // good view
-      S |= 1u << j;
-      psi = psi / (float)nvalid;                   // Eq. (4)
-      pm = (j == v_prev) ? 2.f * psi : psi;        // Eqs. (5), (6)
-    }
+    for (int i = 0; i < kRegions; i++)
+      if (valid >> i & 1u) score.add(a, M[at(8 * j + i)]);
+    float pm;
+    if (score.weigh(a, nvalid, j == v_prev, &pm)) S |= 1u << j;
     psim[at(j)] = pm;
   }
   sh.bits[1][at(w)] = S;
@@ -337,6 +327,7 @@ __device__ __forceinline__ void init_team(const A& a, TeamShared<T>& sh, float* 
                                           int* npairs) {
   const int lane = threadIdx.x & 31;
   const int N = a.N;
+  phase_before_done();                    // launched without overlap: only lets the first phase's blocks in
   const bool live = x < a.W && y < a.H;
   x = min(x, a.W - 1);
   y = min(y, a.H - 1);

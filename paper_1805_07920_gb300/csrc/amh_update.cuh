@@ -545,39 +545,45 @@ struct PixelArrays {
   float M[kRegions * kMaxSrc];
   float w[kMaxSrc];
   float4 C[kRegions];
+  float D[kRegions];          // depth of the propagated planes at the pixel
+  int pick[kRegions];         // their pixels' packed offsets
   __device__ float& m(int g, int j, int) { return M[g * kMaxSrc + j]; }
   __device__ float& wt(int j) { return w[j]; }
   __device__ float4& cc(int g) { return C[g]; }
 };
 
-// Eqs. (2)-(6): weights of the N views from the 8 x N matrix (rows of invalid
-// regions are left out of the counts and of the mean of Eq. (4)).
+// Eqs. (2)-(5) of one view, from its costs as they come (rows of invalid regions
+// are left out of the counts and of the mean of Eq. (4)): counted beside the
+// matrix, because a pass over the finished matrix read it back from the L2 (the
+// blocks of an SM hold 250 KB of local memory against about 100 KB of L1).
+struct ViewScore {
+  int good = 0, bad = 0;
+  float psi = 0.f;
+  template <class A>
+  __device__ __forceinline__ void add(const A& a, float m) {
+    good += m < a.tau;
+    bad += m > a.tau_up;
+    psi += expf(-m * m * a.inv2beta2);             // Eq. (3)
+  }
+  // true: a good view, *pm its psi_mod
+  template <class A>
+  __device__ __forceinline__ bool weigh(const A& a, int nvalid, bool previous, float* pm) {
+    *pm = 0.f;
+    if (!(good > a.n1 && bad < a.n2)) return false;
+    psi = psi / (float)nvalid;                     // Eq. (4)
+    *pm = previous ? 2.f * psi : psi;              // Eqs. (5), (6)
+    return true;
+  }
+};
+
+// Eqs. (4)-(6): weights of the N views from their psi_mod (in w) and the set S
+// of good views.
 template <class A>
 __device__ __forceinline__ void joint_view_selection(const A& a, PixelArrays& sm, uint32_t valid,
-                                                     uint32_t S_prev, int v_prev, uint32_t* S_out, int* v_out) {
+                                                     uint32_t S_prev, uint32_t S, int* v_out) {
   const int N = a.N;
   const int nvalid = __popc(valid);
   const int k = a.k < N ? a.k : N;
-  uint32_t S = 0;
-  for (int j = 0; j < N; j++) {         // psi_mod of the good views into w
-    int ng = 0, nb = 0;
-    float psi = 0.f;
-#pragma unroll
-    for (int i = 0; i < kRegions; i++) {
-      if (!(valid >> i & 1u)) continue;
-      const float m = sm.m(i, j, N);
-      ng += m < a.tau;
-      nb += m > a.tau_up;
-      psi += expf(-m * m * a.inv2beta2);          // Eq. (3)
-    }
-    float pm = 0.f;
-    if (ng > a.n1 && nb < a.n2) {                  // good view
-      S |= 1u << j;
-      psi = psi / (float)nvalid;                   // Eq. (4)
-      pm = (j == v_prev) ? 2.f * psi : psi;        // Eqs. (5), (6)
-    }
-    sm.wt(j) = pm;
-  }
   uint32_t kept = 0;
   int v = -1;
   for (int j = 0; j < N; j++) {
@@ -619,7 +625,6 @@ __device__ __forceinline__ void joint_view_selection(const A& a, PixelArrays& sm
     }
     for (int j = 0; j < N; j++) sm.wt(j) = (low >> j & 1u) ? 1.f : 0.f;
   }
-  *S_out = S;
   *v_out = v;
 }
 
@@ -743,17 +748,16 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
     pick[g] = best;
   }
   }
-  float hD[kRegions];
   uint32_t valid = 0;
 #pragma unroll
   for (int g = 0; g < kRegions; g++) {
-    hD[g] = 0.f;
     if (pick[g] < 0) continue;
     float Dx;
     float4 c;
     if (!propagate(a, a.plane[pick_index(pick[g])], x + (pick[g] & 255) - 32, y + (pick[g] >> 8) - 32, ray, &Dx, &c)) continue;
     sm.cc(g) = c;
-    hD[g] = Dx;
+    sm.D[g] = Dx;
+    sm.pick[g] = pick[g];
     valid |= 1u << g;
   }
 
@@ -763,6 +767,9 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
 
   // --- Eq. (1): the 8 x N cost matrix (views outer: the 8 hypotheses of a view
   // fetch neighbouring texels) -------------------------------------------------------
+  const int nvalid = __popc(valid);
+  const int v_prev = live ? (int)a.vbest[pi] : 255;      // 255: none
+  uint32_t St = 0;                                       // the good views
   if constexpr (kStaged) {
     // one shared-memory box per view for the whole block, placed where a few
     // of the pixels' own planes put their windows
@@ -776,23 +783,34 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
       fill_box(V, ss->box, bp);
       __syncthreads();
       const uint32_t adj = box_adjust(bp);
+      ViewScore score;
 #pragma unroll 1
       for (int g = 0; g < kRegions; g++) {
         const bool ok = valid >> g & 1u;
         const float4 c = ok ? sm.cc(g) : make_float4(0.f, 0.f, 0.f, 0.f);
         const float m = ncc_cost_boxed<kHalf>(V, c, ok, ray, rw, npairs, bp, ss->box, adj);
         if (live) sm.m(g, j, N) = m;
+        if (!(kMode & kHeuristic) && ok) score.add(a, m);
       }
+      float pm;
+      if (!(kMode & kHeuristic) && score.weigh(a, nvalid, j == v_prev, &pm)) St |= 1u << j;
+      if (!(kMode & kHeuristic)) sm.wt(j) = pm;
     }
   } else {
     for (int j = 0; j < N; j++) {
       const ViewConst& V = a.v[j];
+      ViewScore score;
 #pragma unroll 1
       for (int g = 0; g < kRegions; g++) {
         const bool ok = valid >> g & 1u;
         const float4 c = ok ? sm.cc(g) : make_float4(0.f, 0.f, 0.f, 0.f);
-        sm.m(g, j, N) = ncc_cost<kHalf, kTex>(V, c, ok, ray, rw, npairs);
+        const float m = ncc_cost<kHalf, kTex>(V, c, ok, ray, rw, npairs);
+        sm.m(g, j, N) = m;
+        if (!(kMode & kHeuristic) && ok) score.add(a, m);
       }
+      float pm;
+      if (!(kMode & kHeuristic) && score.weigh(a, nvalid, j == v_prev, &pm)) St |= 1u << j;
+      if (!(kMode & kHeuristic)) sm.wt(j) = pm;
     }
   }
 
@@ -805,7 +823,6 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
     for (int j = 0; j < N; j++) sm.wt(j) = ncc_cost<kHalf, kTex>(a.v[j], c, ok, ray, rw, npairs);
     float bm = kbest_mean(sm.w, N, k);
     int choice = 8;
-    float bestD = 0.f;
 #pragma unroll 1
     for (int g = 0; g < kRegions; g++) {
       if (!(valid >> g & 1u)) continue;
@@ -813,10 +830,8 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
       if (r < bm) { bm = r; choice = g; }
     }
     if (choice < 8) {
-#pragma unroll
-      for (int g = 0; g < kRegions; g++) if (g == choice) bestD = hD[g];
-      const float4 pq = a.plane[pick_index(pick[choice])];
-      best = make_float4(pq.x, pq.y, pq.z, bestD);
+      const float4 pq = a.plane[pick_index(sm.pick[choice])];
+      best = make_float4(pq.x, pq.y, pq.z, sm.D[choice]);
     }
     const int nc = a.t < 3 ? 1 : kMaxRefine;
     int bc = -1;
@@ -843,10 +858,8 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
   }
 
   // --- Eqs. (2)-(6) ------------------------------------------------------------------
-  uint32_t St;
   int v;
-  const uint8_t vb = live ? a.vbest[pi] : (uint8_t)255;
-  joint_view_selection(a, sm, valid, live ? a.sel[pi] : 0u, vb == 255 ? -1 : (int)vb, &St, &v);
+  joint_view_selection(a, sm, valid, live ? a.sel[pi] : 0u, St, &v);
   float sw = 0.f;
   uint32_t wm = 0;
   for (int j = 0; j < N; j++) {
@@ -867,7 +880,6 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
   }
   bm *= inv_sw;
   int choice = 8;
-  float bestD = 0.f;
 #pragma unroll 1
   for (int g = 0; g < kRegions; g++) {
     if (!(valid >> g & 1u)) continue;
@@ -880,10 +892,8 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
     if (r < bm) { bm = r; choice = g; }
   }
   if (choice < 8) {
-#pragma unroll
-    for (int g = 0; g < kRegions; g++) if (g == choice) bestD = hD[g];
-    const float4 pq = a.plane[pick_index(pick[choice])];
-    best = make_float4(pq.x, pq.y, pq.z, bestD);
+    const float4 pq = a.plane[pick_index(sm.pick[choice])];
+    best = make_float4(pq.x, pq.y, pq.z, sm.D[choice]);
   }
 
   // --- Sec. 3.3: refinement with the same weights -------------------------------------

@@ -156,19 +156,20 @@ struct FuseArgs {
 // repeated with the correctly rounded operations (check_exactly).
 constexpr float kTiny = 1e-30f, kHuge = 1e30f;
 
-// A block takes 32 x 4 pixels of one view (bands of rows in turn), a warp 32
-// pixels of a row; neighbouring blocks take the same tile of all views, so that
-// what they gather from the other views is in L2 (view after view each of ten
-// 1600 x 1056 views read the others' 270 MB again).  What bounds it: instruction
-// issue, about 200 per check of which 130 are the rounded arithmetic of an
-// agreeing one, then the gathers.  Before, per view pair five correctly rounded
-// divisions and three roots with their branches, the views' constants by
-// indexed loads, a 64-bit division per pixel and 24-byte strided stores: ten
-// 1600 x 1056 views 1670 us, now 1117.  Measured and left: two or four pixels per
-// thread 1566 / 1827 us (registers), the next view's fetches issued ahead 1289,
-// five blocks of 8 warps (48 registers) 1322.  Points leave through shared
-// memory as rows of 768 bytes.
-constexpr int kFuseWarps = 4, kFuseRows = kFuseWarps, kFuseBlocksPerSM = 8;   // 64 registers
+// A block takes 32 x 16 pixels of one view, a warp 32 pixels of a row;
+// neighbouring blocks take the same tile of all views, so that what they gather
+// from the other views is in L2 (view after view, ten 1600 x 1056 views took
+// 1384 us instead of 1171).  What bounds it: instruction issue, about 200 per
+// agreeing check of which 130 are the rounded arithmetic, then the gathers.
+// Before, per view pair five correctly rounded divisions and three roots with
+// their branches, the views' constants by indexed loads, a 64-bit division per
+// pixel and 24-byte strided stores: ten 1600 x 1056 views 1670 us, now 1017; twenty
+// views around a ring, where most checks fail, 8.5 ms, now 7.1 ms.  With four
+// rows instead of 16 per block the set-up of the constants shows: 1116 us and 10.3
+// ms.  Measured and left: two or four pixels per thread 1566 / 1827 us
+// (registers), the next view's fetches issued ahead 1289, five blocks of 8 warps
+// (48 registers) 1322.  Points leave through shared memory as rows of 768 bytes.
+constexpr int kFuseWarps = 4, kFuseRows = 4 * kFuseWarps, kFuseBlocksPerSM = 8;   // 64 registers
 // a view's constants in shared memory, read as float4
 struct FuseShared {
   float4 R[3];          // rows of R, t in w
@@ -176,12 +177,7 @@ struct FuseShared {
   float4 Kinv[3];       // rows of K^-1; in row 0 the baseline to view i times the focal length in w
   const float *depth, *normal;
   int W;
-};
-// One check in flight: z and the numerators of the projection into view j, the
-// pixel (uf, vf) there and what it holds.
-struct FuseCheck {
-  float nu, nv, z, iz, uf, vf, D, m0, m1, m2;
-  bool in, unsure;
+  float lim;            // a pixel coordinate beyond it is outside
 };
 struct FuseExact {
   float uf, vf, D, m0, m1, m2;
@@ -189,20 +185,19 @@ struct FuseExact {
 };
 // The check in full: floor(num / z + 0.5) inside the view, a depth there, the
 // disparity and the angle.
-__device__ __noinline__ FuseExact check_exactly(const float* depth, const float* normal, const FuseShared& S, float nu,
-                                                float nv, float z, float n0, float n1, float n2, float nn, float eps,
-                                                float cos_ang) {
+__device__ __noinline__ FuseExact check_exactly(const FuseShared& S, float nu, float nv, float z, float n0, float n1,
+                                                float n2, float nn, float eps, float cos_ang) {
   FuseExact c = {};
   c.uf = floorf(nu / z + 0.5f);
   c.vf = floorf(nv / z + 0.5f);
   if (!(c.uf >= 0.f && c.uf < S.K[0].w && c.vf >= 0.f && c.vf < S.K[1].w)) return c;
   const size_t q = (size_t)(int)c.vf * S.W + (int)c.uf;
-  c.D = depth[q];
+  c.D = S.depth[q];
   if (!(c.D > 0.f)) return c;
   if (!(S.Kinv[0].w * fabsf(1.f / z - 1.f / c.D) <= eps)) return c;
-  c.m0 = normal[3 * q];
-  c.m1 = normal[3 * q + 1];
-  c.m2 = normal[3 * q + 2];
+  c.m0 = S.normal[3 * q];
+  c.m1 = S.normal[3 * q + 1];
+  c.m2 = S.normal[3 * q + 2];
   const float4 r0 = S.R[0], r1 = S.R[1], r2 = S.R[2];
   const float a0 = r0.x * c.m0 + r1.x * c.m1 + r2.x * c.m2, a1 = r0.y * c.m0 + r1.y * c.m1 + r2.y * c.m2,
               a2 = r0.z * c.m0 + r1.z * c.m1 + r2.z * c.m2;
@@ -221,6 +216,8 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocksPerSM) fuse_kernel
   const int i = (int)(blockIdx.x % (unsigned)a.n), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = (int)(blockIdx.x / (unsigned)a.n);
   const FuseView& Vi = a.v[i];
+  const int x0 = tile % a.tiles_x * 32, px = x0 + lane;
+  if (x0 >= Vi.W || (int64_t)(tile / a.tiles_x) * kFuseRows >= Vi.H) return;   // views smaller than the largest
   if (threadIdx.x < a.n) {
     const FuseView& V = a.v[threadIdx.x];
     FuseShared& S = view[threadIdx.x];
@@ -232,14 +229,16 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocksPerSM) fuse_kernel
       S.Kinv[r] = make_float4(V.Kinv[3 * r], V.Kinv[3 * r + 1], V.Kinv[3 * r + 2],
                               r ? 0.f : V.K[0] * sqrtf(bx * bx + by * by + bz * bz));
     S.W = V.W;
+    S.lim = (float)max(V.W, V.H) + 1.f;
     S.depth = V.depth;
     S.normal = V.normal;
   }
   __syncthreads();
-  const int x0 = tile % a.tiles_x * 32, px = x0 + lane;
-  if (x0 >= Vi.W) return;                    // views smaller than the largest
   const int cols = min(32, Vi.W - x0);
-  for (int64_t row = (int64_t)(tile / a.tiles_x) * kFuseRows + warp; row < Vi.H; row += (int64_t)a.bands * kFuseRows) {
+  // rows of the tile (with fewer bands than the rows need, of every bands-th one)
+  for (int64_t k = warp;; k += kFuseWarps) {
+    const int64_t row = ((int64_t)(tile / a.tiles_x) + k / kFuseRows * a.bands) * kFuseRows + k % kFuseRows;
+    if (row >= Vi.H) break;
     const size_t p = (size_t)row * Vi.W + px;
     const float x = (float)px, y = (float)row;
     const float D = lane < cols ? Vi.depth[p] : 0.f;
@@ -262,70 +261,65 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocksPerSM) fuse_kernel
       float sX[3] = {X[0], X[1], X[2]}, sN[3] = {n[0], n[1], n[2]};
       const float rnn = rcp_approx(nn);
       const bool nn_ok = nn > 1e-5f && nn < 1e5f;
-      // projection into view j and the fetches there
-      auto project = [&](int j, FuseCheck& c) {
+#pragma unroll 1
+      for (int j = 0; j < a.n; j++) {
+        if (j == i) continue;
         const FuseShared& S = view[j];
-        const float4 r0 = S.R[0], r1 = S.R[1], r2 = S.R[2], k0 = S.K[0], k1 = S.K[1];
+        const float4 r0 = S.R[0], r1 = S.R[1], r2 = S.R[2];
+        const float z = r2.x * X[0] + r2.y * X[1] + r2.z * X[2] + r2.w;
+        if (!(z > 0.f)) continue;
+        const float4 k0 = S.K[0], k1 = S.K[1];
         const float X0 = r0.x * X[0] + r0.y * X[1] + r0.z * X[2] + r0.w;
         const float X1 = r1.x * X[0] + r1.y * X[1] + r1.z * X[2] + r1.w;
-        c.z = r2.x * X[0] + r2.y * X[1] + r2.z * X[2] + r2.w;
-        c.iz = rcp_approx(c.z);
-        c.nu = k0.x * X0 + k0.y * X1 + k0.z * c.z;
-        c.nv = k1.x * X0 + k1.y * X1 + k1.z * c.z;
-        const float u = c.nu * c.iz, v = c.nv * c.iz;
-        c.uf = floorf(u + 0.5f);
-        c.vf = floorf(v + 0.5f);
+        const float iz = rcp_approx(z);
+        const float nu = k0.x * X0 + k0.y * X1 + k0.z * z, nv = k1.x * X0 + k1.y * X1 + k1.z * z;
+        const float u = nu * iz, v = nv * iz;
+        float uf = floorf(u + 0.5f), vf = floorf(v + 0.5f);
         // The quotients are within 2^-22 |u| of the rounded ones, whose sums with
         // 0.5 round by 2^-24 (|u| + 0.5): u - uf within 2^-21 (|u| + 1) of -0.5 or
-        // 0.5 leaves the pixel open.
-        const float off = fmaxf(fabsf(u - c.uf), fabsf(v - c.vf));
-        const float m = fmaf(-4.76837158203125e-7f, fmaxf(fabsf(u), fabsf(v)), 0.5f - 4.76837158203125e-7f);
-        const bool z_ok = c.z > kTiny && c.z < kHuge;
-        c.in = z_ok && c.uf >= 0.f && c.uf < k0.w && c.vf >= 0.f && c.vf < k1.w;
-        c.unsure = c.z > 0.f && !(off <= m && z_ok);
-        c.D = 0.f;
-        if (c.in) {
-          const int64_t q = (int64_t)(int)c.vf * S.W + (int)c.uf;
-          const float* ncj = S.normal + 3 * q;
-          c.D = __ldg(S.depth + q);
-          c.m0 = __ldg(ncj);
-          c.m1 = __ldg(ncj + 1);
-          c.m2 = __ldg(ncj + 2);
-        }
-      };
-      auto judge = [&](int j, FuseCheck& c) {
-        const bool has = c.in && c.D > 0.f;
-        if (!has && !c.unsure) return;
-        const FuseShared& S = view[j];
-        const float4 i0 = S.Kinv[0], r0 = S.R[0], r1 = S.R[1], r2 = S.R[2];
-        const float rd = rcp_approx(c.D), dd = fmaf(i0.w, fabsf(c.iz - rd), -a.f_eps);
-        const float md = fmaf(2.384185791015625e-7f * i0.w, c.iz + rd, 1e-6f * a.f_eps);      // 2^-22
-        float nj0 = r0.x * c.m0 + r1.x * c.m1 + r2.x * c.m2, nj1 = r0.y * c.m0 + r1.y * c.m1 + r2.y * c.m2,
-              nj2 = r0.z * c.m0 + r1.z * c.m1 + r2.z * c.m2;
+        // 0.5 leaves the pixel open, unless both images of it lie outside (|u| or
+        // |v| beyond lim, the larger size + 1).
+        const float off = fmaxf(fabsf(u - uf), fabsf(v - vf));
+        const float big = fmaxf(fabsf(u), fabsf(v)), m = fmaf(-4.76837158203125e-7f, big, 0.5f - 4.76837158203125e-7f);
+        const bool z_ok = z > kTiny && z < kHuge;
+        const bool in = z_ok && uf >= 0.f && uf < k0.w && vf >= 0.f && vf < k1.w;
+        bool unsure = (!(off <= m) && big <= S.lim) || !z_ok;
+        if (!in && !unsure) continue;
+        const int64_t q = in ? (int64_t)(int)vf * S.W + (int)uf : 0;
+        const float* ncj = S.normal + 3 * q;
+        float D2 = __ldg(S.depth + q);
+        const float m0 = __ldg(ncj), m1 = __ldg(ncj + 1), m2 = __ldg(ncj + 2);
+        const float4 i0 = S.Kinv[0];
+        const bool has = in && D2 > 0.f;
+        const float rd = rcp_approx(D2), dd = fmaf(i0.w, fabsf(iz - rd), -a.f_eps);
+        const float md = fmaf(2.384185791015625e-7f * i0.w, iz + rd, 1e-6f * a.f_eps);      // 2^-22
+        float nj0 = r0.x * m0 + r1.x * m1 + r2.x * m2, nj1 = r0.y * m0 + r1.y * m1 + r2.y * m2,
+              nj2 = r0.z * m0 + r1.z * m1 + r2.z * m2;
         const float q2 = nj0 * nj0 + nj1 * nj1 + nj2 * nj2;
         const float da = fmaf(n[0] * nj0 + n[1] * nj1 + n[2] * nj2, rsqrt_approx(q2) * rnn, -a.cos_ang);
         bool agree = has && dd <= 0.f && da >= 0.f;
         // sure: the disparity further from the threshold than its error and, if it
         // passes, the cosine too (|cosine| <= 1 + 1e-6: 4e-6 covers its error);
         // comparisons with NaN are not
-        const bool sure = c.D > kTiny && fabsf(dd) > md && (dd > 0.f || (nn_ok && q2 > kTiny && fabsf(da) > 4e-6f));
-        if (c.unsure || (has && !sure)) {
-          const FuseExact e = check_exactly(S.depth, S.normal, S, c.nu, c.nv, c.z, n[0], n[1], n[2], nn, a.f_eps, a.cos_ang);
+        const bool sure = D2 > kTiny && fabsf(dd) > md && (dd > 0.f || (nn_ok && q2 > kTiny && fabsf(da) > 4e-6f));
+        unsure |= has && !sure;
+        if (unsure) {
+          const FuseExact e = check_exactly(S, nu, nv, z, n[0], n[1], n[2], nn, a.f_eps, a.cos_ang);
           agree = e.agree;
-          c.uf = e.uf;
-          c.vf = e.vf;
-          c.D = e.D;
+          uf = e.uf;
+          vf = e.vf;
+          D2 = e.D;
           nj0 = r0.x * e.m0 + r1.x * e.m1 + r2.x * e.m2;
           nj1 = r0.y * e.m0 + r1.y * e.m1 + r2.y * e.m2;
           nj2 = r0.z * e.m0 + r1.z * e.m1 + r2.z * e.m2;
         }
-        if (!agree) return;
+        if (!agree) continue;
         // the agreeing view's own point at q
         const float4 i1 = S.Kinv[1], i2 = S.Kinv[2];
-        const float qx = i0.x * c.uf + i0.y * c.vf + i0.z;
-        const float qy = i1.x * c.uf + i1.y * c.vf + i1.z;
-        const float qz = i2.x * c.uf + i2.y * c.vf + i2.z;
-        const float ex = c.D * qx - r0.w, ey = c.D * qy - r1.w, ez = c.D * qz - r2.w;
+        const float qx = i0.x * uf + i0.y * vf + i0.z;
+        const float qy = i1.x * uf + i1.y * vf + i1.z;
+        const float qz = i2.x * uf + i2.y * vf + i2.z;
+        const float ex = D2 * qx - r0.w, ey = D2 * qy - r1.w, ez = D2 * qz - r2.w;
         sX[0] += r0.x * ex + r1.x * ey + r2.x * ez;
         sX[1] += r0.y * ex + r1.y * ey + r2.y * ez;
         sX[2] += r0.z * ex + r1.z * ey + r2.z * ez;
@@ -333,13 +327,6 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocksPerSM) fuse_kernel
         sN[1] += nj1;
         sN[2] += nj2;
         cnt++;
-      };
-      auto after = [&](int j) { return j + 1 == i ? j + 2 : j + 1; };
-#pragma unroll 1
-      for (int j = i == 0 ? 1 : 0; j < a.n; j = after(j)) {
-        FuseCheck A;
-        project(j, A);
-        judge(j, A);
       }
       if (cnt >= a.f_con) {
         const float inv = 1.f / (float)(1 + cnt);

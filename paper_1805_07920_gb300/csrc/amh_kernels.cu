@@ -18,10 +18,9 @@ using namespace upd;
 constexpr int kTile = 16;
 constexpr int kThreads = 128;
 // 128 registers per thread; the window weights are 36 KB of shared memory per
-// block, so 4 blocks leave about 100 KB of L1.  3200 x 2112, 10 sources, six
-// iterations: 3 blocks 171 ms, 4: 165.5, 5 (96 registers): 165.4, and 5 lost
-// 2 - 5 % on the smaller images (all before the rows ran in two passes, see
-// ncc_window).  The staged sweep's boxes allow 3.
+// block, so 4 blocks leave about 100 KB of L1.  Five blocks (96 registers): the
+// learned form at 1600 x 1056 32.2 ms against 31.9, 640 x 480 3.99 against 3.65.
+// The staged sweep's boxes allow 3.
 constexpr int kPhaseBlocksPerSM = 4, kStagedBlocksPerSM = 3;
 
 // npairs: evaluations of this thread, plus 2^16 for each one sampled from a
@@ -123,7 +122,8 @@ void prefer_carveout(K kernel, int blocks, int smem, std::once_flag* once) {
 // weighs more).  Six sources, four iterations, 1 / 4 / 8 / 16 warps in us:
 // 64x48 750 / 328 / 233 / 229, 160x120 802 / 385 / 324 / 414, 320x240 1143 /
 // 1018 / 1078 / 1474, 400x300 1683 / 1563 / 1635 / 2299, 440x330 1748 / 1880 /
-// 1951 / 2794; with two sources 320x240 takes 462 / 501 / 611 / 972.
+// 1951 / 2794; with two sources 320x240 takes 462 / 501 / 611 / 972 (each phase
+// set up after the one before had ended, see launch_phase_team).
 int team_warps(int groups, int n_src) {
   static int n_sm[64] = {};
   int dev = 0;

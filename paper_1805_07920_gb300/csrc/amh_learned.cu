@@ -7,12 +7,13 @@
 //
 // Kernels: 3x3 convolution forward on the fifth-generation tensor cores
 // (tcgen05.mma, FP32 accumulator in tensor memory, BF16 operands brought in by
-// the tensor memory accelerator; fused bias / ReLU / skip add), the data
-// gradient as the same convolution with flipped, transposed weights, the
-// weight gradient on the same tensor-core path, reading the pixel-major
-// operands directly (amh_conv_tc.cuh; bias gradients in FP32), 2x2 average pooling,
-// nearest upsampling, the L1 loss, Adam, and the feature / head / proposal
-// conversions.
+// the tensor memory accelerator), bias, ReLU, skip addition, 2x2 average pooling
+// and nearest upsampling in its epilogue; the data gradient as the same
+// convolution with flipped, transposed weights, the adjoints of pooling and
+// upsampling, the ReLU masks and the bias sums in its epilogue; the weight
+// gradient on the same tensor-core path, reading the pixel-major operands
+// directly (amh_conv_tc.cuh); the L1 loss, Adam, and the feature / head /
+// proposal conversions.
 //
 // Layout: activations (H, W, C) with C a multiple of 16, BF16 between
 // layers; conv weights (9, Cout, Cin) BF16 (FP32 master copy for Adam), tap

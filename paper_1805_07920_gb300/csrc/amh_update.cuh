@@ -275,8 +275,8 @@ struct RowFetch {
 // ~45 KB and "no instruction" was 12 % of the warps' time at 16 warps per SM.
 // So the rows run in two passes of kRowGroup = 3, 18 fetches in flight before
 // the first is used (about 110 of the 128 registers).  1600 x 1056, 10 sources,
-// five iterations with the proposal: 6 rows unrolled 35.5 ms, 3: 33.5, 2: 34.0,
-// 1: 35.2 (12 warps per SM, weights in registers, everything unrolled: 38.0).
+// five iterations with the proposal: 6 rows unrolled 33.5 ms, 3: 31.9, 2: 33.0
+// (12 warps per SM, weights in registers, everything unrolled: 38.0 before).
 constexpr int kRowGroup = 3;
 static_assert(kWinN % kRowGroup == 0, "the rows of a window are processed in whole groups");
 template <bool kHalf, int kFetch, class Win>

@@ -52,3 +52,28 @@ def test_team_sizes(amh, synth_mod, form):
 def test_team_sources(amh, synth_mod, n_src, k):
     sc = synth_mod.scene_many(seed=7)
     _compare(amh, sc.cams, sc.images, [sc.ref], [sc.src[:n_src]], 4, k=k)
+
+
+def test_team_launches_in_a_graph(amh, synth_mod):
+    """The overlapped launches of small images under stream capture: replays of
+    the captured initialisation and iterations equal direct calls."""
+    import ctypes
+    import torch
+    sc = synth_mod.make_scene("tiny")
+    g = amh.Context.from_scene(sc, seed=21)
+    g.init_random()
+    g.iterate(4)
+    want = g.get_state()
+    s = torch.cuda.Stream()
+    g.set_stream(ctypes.c_void_p(s.cuda_stream))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        g.init_random()
+        g.iterate(4)
+    for _ in range(2):
+        graph.replay()
+        torch.cuda.synchronize()
+        got = g.get_state()
+        for k in KEYS:
+            np.testing.assert_array_equal(got[k], want[k], err_msg=k)

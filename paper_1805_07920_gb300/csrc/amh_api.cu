@@ -177,10 +177,11 @@ AMH_API int amh_create(amh_ctx** out, const amh_params* p, int32_t n_views, cons
   c->p = *p;
   c->ref = ref;
   {
-    const cudaError_t e = cudaGetDevice(&c->device);
+    cudaError_t e = cudaGetDevice(&c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) {
       delete c;
-      return fail(nullptr, AMH_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
+      return fail(nullptr, AMH_ECUDA, "current device: %s", cudaGetErrorString(e));
     }
   }
   c->N = n_src;
@@ -400,7 +401,7 @@ AMH_API int amh_init_random(amh_ctx* c) {
   if (!c) return AMH_EINVAL;
   c->t = 0;
   fill_step_args(c, 0);
-  launch_init(c->args, c->stream);
+  launch_init(c->args, c->n_sm, c->stream);
   int rc = launch_check(c, "init");
   if (rc) return rc;
   c->initialized = true;
@@ -412,7 +413,7 @@ AMH_API int amh_step_phase(amh_ctx* c, int32_t color) {
   if (color != 0 && color != 1) return fail(c, AMH_EINVAL, "color must be 0 or 1");
   if (!c->initialized) return fail(c, AMH_ESTATE, "state not initialised (amh_init_random or amh_set_state)");
   fill_step_args(c, color);
-  launch_phase(c->args, c->stream);
+  launch_phase(c->args, c->n_sm, c->stream);
   int rc = launch_check(c, "phase");
   if (rc) return rc;
   if (color == 1) c->t++;

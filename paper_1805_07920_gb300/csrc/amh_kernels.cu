@@ -124,12 +124,8 @@ void prefer_carveout(K kernel, int blocks, int smem, std::once_flag* once) {
 // 1018 / 1078 / 1474, 400x300 1683 / 1563 / 1635 / 2299, 440x330 1748 / 1880 /
 // 1951 / 2794; with two sources 320x240 takes 462 / 501 / 611 / 972 (each phase
 // set up after the one before had ended, see launch_phase_team).
-int team_warps(int groups, int n_src) {
-  static int n_sm[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (!n_sm[dev & 63]) cudaDeviceGetAttribute(&n_sm[dev & 63], cudaDevAttrMultiProcessorCount, dev);
-  const int warps = 16 * n_sm[dev & 63];
+int team_warps(int groups, int n_src, int n_sm) {
+  const int warps = 16 * n_sm;
   if (groups * 16 <= warps) return 16;
   if (groups * 8 <= warps) return 8;
   return groups * 10 <= warps * (n_src < 4 ? 4 : 8) ? 4 : 1;
@@ -173,9 +169,9 @@ int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
 }
 
 template <bool kHalf, bool kTex>
-int launch_init_t(const PhaseArgs& a, cudaStream_t s) {
+int launch_init_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
   static std::once_flag once[64];
-  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N)) {
+  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N, n_sm)) {
     case 16: return launch_init_team<kHalf, kTex, 16>(a, s);
     case 8: return launch_init_team<kHalf, kTex, 8>(a, s);
     case 4: return launch_init_team<kHalf, kTex, 4>(a, s);
@@ -188,16 +184,16 @@ int launch_init_t(const PhaseArgs& a, cudaStream_t s) {
 }
 // the texture-filter form exists for uint8 images only (the context refuses
 // it with FP16 images and with the ablations)
-int launch_init(const PhaseArgs& a, cudaStream_t s) {
-  if (a.tex_filter) return launch_init_t<false, true>(a, s);
-  return a.img_half ? launch_init_t<true, false>(a, s) : launch_init_t<false, false>(a, s);
+int launch_init(const PhaseArgs& a, int n_sm, cudaStream_t s) {
+  if (a.tex_filter) return launch_init_t<false, true>(a, n_sm, s);
+  return a.img_half ? launch_init_t<true, false>(a, n_sm, s) : launch_init_t<false, false>(a, n_sm, s);
 }
 
 template <bool kHalf, int kMode>
-int launch_phase_t(const PhaseArgs& a, cudaStream_t s) {
+int launch_phase_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
   static std::once_flag once[64];
   if constexpr (kMode == 0 || kMode == kTexture) {   // the ablations and the staged sweep: one thread per pixel
-    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N)) {
+    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N, n_sm)) {
       case 16: return launch_phase_team<kHalf, kMode == kTexture, 16>(a, s);
       case 8: return launch_phase_team<kHalf, kMode == kTexture, 8>(a, s);
       case 4: return launch_phase_team<kHalf, kMode == kTexture, 4>(a, s);
@@ -212,23 +208,23 @@ int launch_phase_t(const PhaseArgs& a, cudaStream_t s) {
   return (int)cudaGetLastError();
 }
 template <int kMode>
-int launch_phase_m(const PhaseArgs& a, cudaStream_t s) {
+int launch_phase_m(const PhaseArgs& a, int n_sm, cudaStream_t s) {
   // staged sweep on request; at t = 0 the planes are the random ones of the
   // initialisation and no window set fits a box, so those phases fetch
   // through the texture unit
   if (a.staged && a.t > 0)
-    return a.img_half ? launch_phase_t<true, kMode | kStage>(a, s) : launch_phase_t<false, kMode | kStage>(a, s);
-  return a.img_half ? launch_phase_t<true, kMode>(a, s) : launch_phase_t<false, kMode>(a, s);
+    return a.img_half ? launch_phase_t<true, kMode | kStage>(a, n_sm, s) : launch_phase_t<false, kMode | kStage>(a, n_sm, s);
+  return a.img_half ? launch_phase_t<true, kMode>(a, n_sm, s) : launch_phase_t<false, kMode>(a, n_sm, s);
 }
 // the method, or one of the ablations of Sec. 4 (a.ablation: bit 0 symmetric
 // propagation, bit 1 heuristic view selection)
-int launch_phase(const PhaseArgs& a, cudaStream_t s) {
-  if (a.tex_filter) return launch_phase_t<false, kTexture>(a, s);
+int launch_phase(const PhaseArgs& a, int n_sm, cudaStream_t s) {
+  if (a.tex_filter) return launch_phase_t<false, kTexture>(a, n_sm, s);
   switch (a.ablation & 3) {
-    case kSymmetric: return launch_phase_m<kSymmetric>(a, s);
-    case kHeuristic: return launch_phase_m<kHeuristic>(a, s);
-    case kSymmetric | kHeuristic: return launch_phase_m<kSymmetric | kHeuristic>(a, s);
-    default: return launch_phase_m<0>(a, s);
+    case kSymmetric: return launch_phase_m<kSymmetric>(a, n_sm, s);
+    case kHeuristic: return launch_phase_m<kHeuristic>(a, n_sm, s);
+    case kSymmetric | kHeuristic: return launch_phase_m<kSymmetric | kHeuristic>(a, n_sm, s);
+    default: return launch_phase_m<0>(a, n_sm, s);
   }
 }
 

@@ -109,8 +109,9 @@ void fill_step_args(amh_ctx* c, int color) {
   a.tau = (float)(c->p.tau_mc_init * std::exp(-(double)c->t * c->t / (double)c->p.alpha));
 }
 
-int launch_check(amh_ctx* c, const char* what) {
-  cudaError_t e = cudaGetLastError();
+// e: what the launcher returned (it has taken the error off the runtime's record)
+int launch_check(amh_ctx* c, const char* what, int err) {
+  const cudaError_t e = (cudaError_t)err;
   if (e != cudaSuccess) return fail(c, AMH_ECUDA, "%s launch: %s", what, cudaGetErrorString(e));
   return AMH_OK;
 }
@@ -401,8 +402,7 @@ AMH_API int amh_init_random(amh_ctx* c) {
   if (!c) return AMH_EINVAL;
   c->t = 0;
   fill_step_args(c, 0);
-  launch_init(c->args, c->n_sm, c->stream);
-  int rc = launch_check(c, "init");
+  const int rc = launch_check(c, "init", launch_init(c->args, c->n_sm, c->stream));
   if (rc) return rc;
   c->initialized = true;
   return AMH_OK;
@@ -413,8 +413,7 @@ AMH_API int amh_step_phase(amh_ctx* c, int32_t color) {
   if (color != 0 && color != 1) return fail(c, AMH_EINVAL, "color must be 0 or 1");
   if (!c->initialized) return fail(c, AMH_ESTATE, "state not initialised (amh_init_random or amh_set_state)");
   fill_step_args(c, color);
-  launch_phase(c->args, c->n_sm, c->stream);
-  int rc = launch_check(c, "phase");
+  const int rc = launch_check(c, "phase", launch_phase(c->args, c->n_sm, c->stream));
   if (rc) return rc;
   if (color == 1) c->t++;
   return AMH_OK;

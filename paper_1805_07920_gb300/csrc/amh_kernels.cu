@@ -165,7 +165,8 @@ int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return (int)cudaLaunchKernelEx(&cfg, phase_team_kernel<kHalf, kTex, T>, a);
+  cudaLaunchKernelEx(&cfg, phase_team_kernel<kHalf, kTex, T>, a);
+  return (int)cudaGetLastError();
 }
 
 template <bool kHalf, bool kTex>

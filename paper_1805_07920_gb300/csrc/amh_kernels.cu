@@ -49,8 +49,9 @@ __global__ void __launch_bounds__(kThreads, (kMode & kStage) ? kStagedBlocksPerS
     const int y = blockIdx.y * kTile + 4 * (tid >> 5) + 2 * (q >> 1) + ((lane >> 2) & 1);
     const int x = blockIdx.x * kTile + 2 * (4 * (q & 1) + (lane & 3)) + ((y + a.color) & 1);
     // the whole block takes part in the staged sweep, pixels outside the image too
-    __shared__ StageShared ss;
-    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H, &ss);
+    extern __shared__ __align__(16) unsigned char stage_dyn[];
+    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H,
+                               reinterpret_cast<StageShared*>(stage_dyn));
   } else {
     const int y = blockIdx.y * kTile + (tid >> 3);
     const int x = blockIdx.x * kTile + 2 * (tid & 7) + ((y + a.color) & 1);
@@ -130,20 +131,20 @@ int team_warps(int groups, int n_src, int n_sm) {
   if (groups * 8 <= warps) return 8;
   return groups * 10 <= warps * (n_src < 4 ? 4 : 8) ? 4 : 1;
 }
-// the team kernels' dynamic shared memory goes past the default limit with
-// many views; set once per device
+// Static and dynamic shared memory together go past the default limit of 48 KB:
+// the team kernels' with many views, the staged sweep's boxes beside the window
+// weights.  Allowed once per device.
 template <typename K>
-void allow_dynamic(K kernel, std::once_flag* once) {
+void allow_dynamic(K kernel, int bytes, std::once_flag* once) {
   int dev = 0;
   cudaGetDevice(&dev);
-  std::call_once(once[dev & 63], [=] {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, team_floats(kMaxSrc) * (int)sizeof(float));
-  });
+  std::call_once(once[dev & 63], [=] { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
+constexpr int kTeamDynamic = team_floats(kMaxSrc) * (int)sizeof(float);   // most of a team kernel
 template <bool kHalf, bool kTex, int T>
 int launch_init_team(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
-  allow_dynamic(init_team_kernel<kHalf, kTex, T>, once);
+  allow_dynamic(init_team_kernel<kHalf, kTex, T>, kTeamDynamic, once);
   const dim3 grid((a.W + 7) / 8, (a.H + 3) / 4);
   init_team_kernel<kHalf, kTex, T><<<grid, 32 * T, kTeamPixels * a.N * sizeof(float), s>>>(a);
   return (int)cudaGetLastError();
@@ -151,7 +152,7 @@ int launch_init_team(const PhaseArgs& a, cudaStream_t s) {
 template <bool kHalf, bool kTex, int T>
 int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
   static std::once_flag once[64];
-  allow_dynamic(phase_team_kernel<kHalf, kTex, T>, once);
+  allow_dynamic(phase_team_kernel<kHalf, kTex, T>, kTeamDynamic, once);
   const dim3 grid((a.W + 15) / 16, (a.H + 3) / 4);
   // Small phases are short (10 - 20 us): the next one's blocks start loading their
   // windows while this one's last blocks run.
@@ -192,7 +193,7 @@ int launch_init(const PhaseArgs& a, int n_sm, cudaStream_t s) {
 
 template <bool kHalf, int kMode>
 int launch_phase_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
-  static std::once_flag once[64];
+  static std::once_flag once[2][64];
   if constexpr (kMode == 0 || kMode == kTexture) {   // the ablations and the staged sweep: one thread per pixel
     switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N, n_sm)) {
       case 16: return launch_phase_team<kHalf, kMode == kTexture, 16>(a, s);
@@ -202,10 +203,12 @@ int launch_phase_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
     }
   }
   constexpr bool kStaged = (kMode & kStage) != 0;
+  constexpr int kDynamic = kStaged ? (int)sizeof(StageShared) : 0;
+  if constexpr (kStaged) allow_dynamic(phase_kernel<kHalf, kMode>, kDynamic, once[1]);
   prefer_carveout(phase_kernel<kHalf, kMode>, kStaged ? kStagedBlocksPerSM : kPhaseBlocksPerSM,
-                  (int)(sizeof(WinShared) + (kStaged ? sizeof(StageShared) : 0)), once);
+                  (int)sizeof(WinShared) + kDynamic, once[0]);
   dim3 grid((a.W + kTile - 1) / kTile, (a.H + kTile - 1) / kTile);
-  phase_kernel<kHalf, kMode><<<grid, kThreads, 0, s>>>(a);
+  phase_kernel<kHalf, kMode><<<grid, kThreads, kDynamic, s>>>(a);
   return (int)cudaGetLastError();
 }
 template <int kMode>

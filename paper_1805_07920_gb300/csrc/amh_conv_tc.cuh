@@ -849,5 +849,17 @@ inline ConvPlan conv_plan(int cin, int cout) {
   return p;
 }
 
+// CTAs of a convolution along its tiles: per channel block (nblk of them) as
+// many as are resident at once, at most one per tile (or pair of tiles).  The
+// gradients' CTAs write four rows of bias partial sums each and have kBiasRows
+// of them; with fewer CTAs each takes more tiles.
+constexpr int kBiasRows = 2048;
+__host__ constexpr int conv_grid(int ntiles, int n_sm, int ctas_per_sm, int nblk, bool gradient) {
+  int g = n_sm * ctas_per_sm / nblk;
+  if (gradient && g > kBiasRows / 4) g = kBiasRows / 4;
+  if (g > ntiles) g = ntiles;
+  return g < 1 ? 1 : g;
+}
+
 }  // namespace tc
 }  // namespace amh

@@ -50,7 +50,7 @@ constexpr LayerDef kNet[kLayers] = {{16, 32, 1}, {32, 64, 1}, {64, 96, 1}, {96, 
 
 // Bias gradients: db of a layer is the sum of the rows of its partial sums
 // (written by the kernels that produce dy), one block per channel and layer.
-constexpr int kBiasRows = 2048;       // most rows of partial sums of a layer
+using tc::kBiasRows;                  // most rows of partial sums of a layer
 struct BiasArgs {
   const float* part[kLayers];
   float* db[kLayers];
@@ -517,7 +517,7 @@ int plan_conv(amh_net* n, ConvOp& op, const __nv_bfloat16* x, const __nv_bfloat1
   const int by_regs = 65536 / (((fa.numRegs + 7) & ~7) * op.threads);
   const int cps = std::max(1, std::min(p.ctas_per_sm, by_regs));
   const int nblk = Cout / p.Nb, ntiles = a.rows * ((W + tc::kM - 1) / tc::kM) / (tc::epi_row_pairs(epi) ? 2 : 1);
-  op.grid = dim3(std::max(1, std::min(ntiles, n_sm * cps / nblk)), nblk);
+  op.grid = dim3(tc::conv_grid(ntiles, n_sm, cps, nblk, tc::epi_gradient(epi)), nblk);
   return AMH_OK;
 }
 int conv(amh_net* n, ConvOp& op, bool overlap) {
@@ -583,7 +583,6 @@ int plan_network(amh_net* n) {
     a.bpart = n->bpart[d[L].to];
     rc = plan_conv(n, n->dgr[L], n->dy16[L], n->wd16[L], f[L].H, f[L].W, kNet[L].cout, kNet[L].cin, d[L].epi, a);
     n->brows[d[L].to] = 4 * (int)n->dgr[L].grid.x;
-    if (!rc && n->brows[d[L].to] > kBiasRows) rc = nfail(n, AMH_EINVAL, "conv: more partial sums than rows");
   }
   // band b of the last layer: rows [H0 b / n, H0 (b + 1) / n); of the layer before
   // it: the rows those need that no earlier band computed (one row ahead)

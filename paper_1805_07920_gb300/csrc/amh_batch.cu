@@ -14,6 +14,7 @@
 // kernels (amh_update.cuh).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -25,6 +26,7 @@
 #include "amh.h"
 #include "amh_device.cuh"
 #include "amh_kernels.h"
+#include "amh_launch.h"
 #include "amh_update.cuh"
 
 namespace amh {
@@ -205,7 +207,7 @@ struct amh_batch {
   int variant = 0;                        // index into kVariants
   int t = 0;
   bool initialized = false;
-  int grid_blocks = 0;
+  DeviceShape dev;
   cudaGraphExec_t graph_exec = nullptr;
   int graph_iters = -1, graph_variant = -1;
   std::string err;
@@ -296,17 +298,37 @@ BatchArgs make_args(amh_batch* b, const RefArgs* refs, int n_items, int color) {
   return a;
 }
 
+// A launch over the work items: persistent blocks, but no more than there are
+// items -- the blocks race for them, and with more blocks than items some SMs take
+// several while others take none.  Four iterations in us, with 608 blocks (four
+// per SM) for any batch and now: three references of 128 x 96 with two sources
+// 753 -> 435, four of 200 x 150 with two 822 -> 691, four of 280 x 200 with two
+// 1266 -> 1189 (617, 722 and 1198 with the window weights in registers and 456
+// blocks).
+template <typename K>
+void launch_items(amh_batch* b, K kernel, const BatchArgs& a) {
+  const int per_sm = blocks_per_sm(a.n_items, b->dev.n_sm, kBBlocksPerSM);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(std::min(a.n_items, per_sm * b->dev.n_sm));
+  cfg.blockDim = dim3(kBThreads);
+  cfg.stream = b->stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at.val.sharedMemCarveout = carveout_percent(per_sm, (int)(sizeof(RefArgs) + sizeof(WinShared)) + 8, b->dev.smem_sm);
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, a);
+}
 template <bool kHalf, int kMode>
 void launch_batch_phase(amh_batch* b, int color) {
   const BatchArgs a = make_args(b, b->d_refs[b->variant], b->items[b->variant], color);
   cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned int), b->stream);
-  const dim3 g(b->grid_blocks), t(kBThreads);
   switch (b->variant) {
-    case 0: batch_phase_kernel<kHalf, 16, 8, kMode><<<g, t, 0, b->stream>>>(a); break;
-    case 1: batch_phase_kernel<kHalf, 32, 16, kMode><<<g, t, 0, b->stream>>>(a); break;
-    case 2: batch_phase_kernel<kHalf, 64, 32, kMode><<<g, t, 0, b->stream>>>(a); break;
-    case 3: batch_phase_kernel<kHalf, 16, 4, kMode><<<g, t, 0, b->stream>>>(a); break;
-    default: batch_phase_kernel<kHalf, 32, 8, kMode><<<g, t, 0, b->stream>>>(a); break;
+    case 0: launch_items(b, batch_phase_kernel<kHalf, 16, 8, kMode>, a); break;
+    case 1: launch_items(b, batch_phase_kernel<kHalf, 32, 16, kMode>, a); break;
+    case 2: launch_items(b, batch_phase_kernel<kHalf, 64, 32, kMode>, a); break;
+    case 3: launch_items(b, batch_phase_kernel<kHalf, 16, 4, kMode>, a); break;
+    default: launch_items(b, batch_phase_kernel<kHalf, 32, 8, kMode>, a); break;
   }
 }
 // FP16 images, uint8 images, or uint8 images through the texture unit's
@@ -324,9 +346,9 @@ int batch_init(amh_batch* b) {
   b->t = 0;
   const BatchArgs a = make_args(b, b->d_refs_init, b->init_items, 0);
   cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned int), b->stream);
-  if (b->tex_filter) batch_init_kernel<false, true><<<b->grid_blocks, kBThreads, 0, b->stream>>>(a);
-  else if (b->half) batch_init_kernel<true, false><<<b->grid_blocks, kBThreads, 0, b->stream>>>(a);
-  else batch_init_kernel<false, false><<<b->grid_blocks, kBThreads, 0, b->stream>>>(a);
+  if (b->tex_filter) launch_items(b, batch_init_kernel<false, true>, a);
+  else if (b->half) launch_items(b, batch_init_kernel<true, false>, a);
+  else launch_items(b, batch_init_kernel<false, false>, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return bfail(b, AMH_ECUDA, "batch init launch: %s", cudaGetErrorString(e));
   b->initialized = true;
@@ -546,10 +568,10 @@ AMH_API int amh_batch_create(amh_batch** out, const amh_params* p, int32_t n_vie
   for (int vi = 0; vi < AMH_BATCH_VARIANTS; vi++)
     CB(upload(kVariants[vi].tw, 2 * kBThreads / kVariants[vi].tw, &b->d_refs[vi], &b->items[vi]));
   CB(upload(16, 8, &b->d_refs_init, &b->init_items));
-  int dev = 0, sms = 0;
+  int dev = 0;
   CB(cudaGetDevice(&dev));
-  CB(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  b->grid_blocks = sms * kBBlocksPerSM;
+  CB(cudaDeviceGetAttribute(&b->dev.n_sm, cudaDevAttrMultiProcessorCount, dev));
+  CB(cudaDeviceGetAttribute(&b->dev.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
   CB(cudaStreamSynchronize(b->stream));
 #undef CB
   *out = b;

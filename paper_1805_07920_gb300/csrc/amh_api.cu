@@ -179,7 +179,9 @@ AMH_API int amh_create(amh_ctx** out, const amh_params* p, int32_t n_views, cons
   c->ref = ref;
   {
     cudaError_t e = cudaGetDevice(&c->device);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->dev.n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    if (e == cudaSuccess)
+      e = cudaDeviceGetAttribute(&c->dev.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device);
     if (e != cudaSuccess) {
       delete c;
       return fail(nullptr, AMH_ECUDA, "current device: %s", cudaGetErrorString(e));
@@ -402,7 +404,7 @@ AMH_API int amh_init_random(amh_ctx* c) {
   if (!c) return AMH_EINVAL;
   c->t = 0;
   fill_step_args(c, 0);
-  const int rc = launch_check(c, "init", launch_init(c->args, c->n_sm, c->stream));
+  const int rc = launch_check(c, "init", launch_init(c->args, c->dev, c->stream));
   if (rc) return rc;
   c->initialized = true;
   return AMH_OK;
@@ -413,7 +415,7 @@ AMH_API int amh_step_phase(amh_ctx* c, int32_t color) {
   if (color != 0 && color != 1) return fail(c, AMH_EINVAL, "color must be 0 or 1");
   if (!c->initialized) return fail(c, AMH_ESTATE, "state not initialised (amh_init_random or amh_set_state)");
   fill_step_args(c, color);
-  const int rc = launch_check(c, "phase", launch_phase(c->args, c->n_sm, c->stream));
+  const int rc = launch_check(c, "phase", launch_phase(c->args, c->dev, c->stream));
   if (rc) return rc;
   if (color == 1) c->t++;
   return AMH_OK;

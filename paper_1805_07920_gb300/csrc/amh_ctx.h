@@ -7,12 +7,13 @@
 
 #include "amh.h"
 #include "amh_device.cuh"
+#include "amh_launch.h"
 
 struct amh_ctx {
   amh_params p;
   int W = 0, H = 0, N = 0, ref = 0;
   int device = 0;                         // the CUDA device current at amh_create
-  int n_sm = 0;                           // and its multiprocessors
+  amh::DeviceShape dev;                   // and its shape
   int src[AMH_MAX_SRC];
   cudaStream_t stream = nullptr;
   cudaArray_t arr[AMH_MAX_SRC] = {};      // source views, uint8 texture arrays

@@ -20,8 +20,9 @@ constexpr int kThreads = 128;
 // 128 registers per thread; the window weights are 36 KB of shared memory per
 // block, so 4 blocks leave about 100 KB of L1.  Five blocks (96 registers): the
 // learned form at 1600 x 1056 32.2 ms against 31.9, 640 x 480 3.99 against 3.65.
-// The staged sweep's boxes allow 3.
-constexpr int kPhaseBlocksPerSM = 4, kStagedBlocksPerSM = 3;
+// The staged sweep's boxes and the window weights in registers (168) allow 3.
+constexpr int kPhaseBlocksPerSM = 4, kThreeBlocksPerSM = 3;
+constexpr int phase_blocks_per_sm(int mode) { return mode & (kStage | kRegs) ? kThreeBlocksPerSM : kPhaseBlocksPerSM; }
 
 // npairs: evaluations of this thread, plus 2^16 for each one sampled from a
 // shared-memory box (fewer than 2^11 per thread and launch); the two totals
@@ -35,12 +36,16 @@ __device__ __forceinline__ void count_pairs(const PhaseArgs& a, int npairs) {
 }
 
 template <bool kHalf, int kMode>
-__global__ void __launch_bounds__(kThreads, (kMode & kStage) ? kStagedBlocksPerSM : kPhaseBlocksPerSM) phase_kernel(const __grid_constant__ PhaseArgs a) {
+__global__ void __launch_bounds__(kThreads, phase_blocks_per_sm(kMode)) phase_kernel(const __grid_constant__ PhaseArgs a) {
   PixelArrays sm;
-  __shared__ WinShared ws;
   const int tid = threadIdx.x;
   int npairs = 0;
-  if constexpr ((kMode & kStage) != 0) {
+  if constexpr ((kMode & kRegs) != 0) {
+    const int y = blockIdx.y * kTile + (tid >> 3);
+    const int x = blockIdx.x * kTile + 2 * (tid & 7) + ((y + a.color) & 1);
+    update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, nullptr, nullptr, x < a.W && y < a.H);
+  } else if constexpr ((kMode & kStage) != 0) {
+    __shared__ WinShared ws;
     // Warp w updates rows 4w .. 4w + 3 of the tile (8 pixels of the colour
     // per row); each quarter-warp takes 4 pixels of two neighbouring rows, so
     // the 8 lanes of a 16-byte shared load sample 8 distinct columns modulo
@@ -53,6 +58,7 @@ __global__ void __launch_bounds__(kThreads, (kMode & kStage) ? kStagedBlocksPerS
     update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H,
                                reinterpret_cast<StageShared*>(stage_dyn));
   } else {
+    __shared__ WinShared ws;
     const int y = blockIdx.y * kTile + (tid >> 3);
     const int x = blockIdx.x * kTile + 2 * (tid & 7) + ((y + a.color) & 1);
     update_pixel<kHalf, kMode>(a, sm, x, y, &npairs, ws.q + tid, ws.slots[tid >> 5], x < a.W && y < a.H);
@@ -97,21 +103,25 @@ __global__ void __launch_bounds__(32 * T, kTeamBlocksPerSM<T>) init_team_kernel(
 
 }  // namespace
 
-// Ask for the smallest shared-memory carve-out that holds `blocks` blocks of
-// `smem` bytes (and the 1 KB each that the system keeps): the rest of the
-// unified L1 is texture and local-memory cache.  The preference is per device,
-// so it is set once for each device that launches the kernel.
+// A launch of one thread per pixel, with the carve-out for the blocks an SM gets.
+// Four iterations in us, with the carve-out for all four blocks and now: two
+// sources 320 x 240 447 -> 430, three 520 x 390 1494 -> 1430; the same at full size.
 template <typename K>
-void prefer_carveout(K kernel, int blocks, int smem, std::once_flag* once) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::call_once(once[dev & 63], [=] {
-    int smem_sm = 0;
-    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const int need = blocks * (smem + 1024);
-    const int pct = smem_sm > 0 ? std::min(100, (100 * need + smem_sm - 1) / smem_sm) : 100;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  });
+int launch_blocks(K kernel, dim3 grid, int most, int smem, int dynamic, const PhaseArgs& a, const DeviceShape& dev,
+                  cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = dynamic;
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at.val.sharedMemCarveout =
+      carveout_percent(blocks_per_sm((int64_t)grid.x * grid.y, dev.n_sm, most), smem + dynamic, dev.smem_sm);
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, a);
+  return (int)cudaGetLastError();
 }
 
 // Warps per 32 pixels for a launch over `groups` groups of 32 pixels: 16, 8 or 4
@@ -171,64 +181,65 @@ int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
 }
 
 template <bool kHalf, bool kTex>
-int launch_init_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
-  static std::once_flag once[64];
-  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N, n_sm)) {
+int launch_init_t(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
+  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N, dev.n_sm)) {
     case 16: return launch_init_team<kHalf, kTex, 16>(a, s);
     case 8: return launch_init_team<kHalf, kTex, 8>(a, s);
     case 4: return launch_init_team<kHalf, kTex, 4>(a, s);
     default: break;
   }
-  prefer_carveout(init_kernel<kHalf, kTex>, kPhaseBlocksPerSM, (int)sizeof(WinShared), once);
-  dim3 grid((a.W + kTile - 1) / kTile, (a.H + 7) / 8);
-  init_kernel<kHalf, kTex><<<grid, kThreads, 0, s>>>(a);
-  return (int)cudaGetLastError();
+  const dim3 grid((a.W + kTile - 1) / kTile, (a.H + 7) / 8);
+  return launch_blocks(init_kernel<kHalf, kTex>, grid, kPhaseBlocksPerSM, (int)sizeof(WinShared), 0, a, dev, s);
 }
 // the texture-filter form exists for uint8 images only (the context refuses
 // it with FP16 images and with the ablations)
-int launch_init(const PhaseArgs& a, int n_sm, cudaStream_t s) {
-  if (a.tex_filter) return launch_init_t<false, true>(a, n_sm, s);
-  return a.img_half ? launch_init_t<true, false>(a, n_sm, s) : launch_init_t<false, false>(a, n_sm, s);
+int launch_init(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
+  if (a.tex_filter) return launch_init_t<false, true>(a, dev, s);
+  return a.img_half ? launch_init_t<true, false>(a, dev, s) : launch_init_t<false, false>(a, dev, s);
 }
 
 template <bool kHalf, int kMode>
-int launch_phase_t(const PhaseArgs& a, int n_sm, cudaStream_t s) {
-  static std::once_flag once[2][64];
+int launch_phase_t(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
   if constexpr (kMode == 0 || kMode == kTexture) {   // the ablations and the staged sweep: one thread per pixel
-    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N, n_sm)) {
+    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N, dev.n_sm)) {
       case 16: return launch_phase_team<kHalf, kMode == kTexture, 16>(a, s);
       case 8: return launch_phase_team<kHalf, kMode == kTexture, 8>(a, s);
       case 4: return launch_phase_team<kHalf, kMode == kTexture, 4>(a, s);
       default: break;
     }
   }
+  const dim3 grid((a.W + kTile - 1) / kTile, (a.H + kTile - 1) / kTile);
+  if constexpr (kMode == kTexture) {
+    if (registers_pay((int64_t)grid.x * grid.y, dev.n_sm, kThreeBlocksPerSM, kPhaseBlocksPerSM))
+      return launch_blocks(phase_kernel<kHalf, kMode | kRegs>, grid, kThreeBlocksPerSM, 0, 0, a, dev, s);
+  }
   constexpr bool kStaged = (kMode & kStage) != 0;
   constexpr int kDynamic = kStaged ? (int)sizeof(StageShared) : 0;
-  if constexpr (kStaged) allow_dynamic(phase_kernel<kHalf, kMode>, kDynamic, once[1]);
-  prefer_carveout(phase_kernel<kHalf, kMode>, kStaged ? kStagedBlocksPerSM : kPhaseBlocksPerSM,
-                  (int)sizeof(WinShared) + kDynamic, once[0]);
-  dim3 grid((a.W + kTile - 1) / kTile, (a.H + kTile - 1) / kTile);
-  phase_kernel<kHalf, kMode><<<grid, kThreads, kDynamic, s>>>(a);
-  return (int)cudaGetLastError();
+  if constexpr (kStaged) {
+    static std::once_flag once[64];
+    allow_dynamic(phase_kernel<kHalf, kMode>, kDynamic, once);
+  }
+  return launch_blocks(phase_kernel<kHalf, kMode>, grid, phase_blocks_per_sm(kMode), (int)sizeof(WinShared), kDynamic, a,
+                       dev, s);
 }
 template <int kMode>
-int launch_phase_m(const PhaseArgs& a, int n_sm, cudaStream_t s) {
+int launch_phase_m(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
   // staged sweep on request; at t = 0 the planes are the random ones of the
   // initialisation and no window set fits a box, so those phases fetch
   // through the texture unit
   if (a.staged && a.t > 0)
-    return a.img_half ? launch_phase_t<true, kMode | kStage>(a, n_sm, s) : launch_phase_t<false, kMode | kStage>(a, n_sm, s);
-  return a.img_half ? launch_phase_t<true, kMode>(a, n_sm, s) : launch_phase_t<false, kMode>(a, n_sm, s);
+    return a.img_half ? launch_phase_t<true, kMode | kStage>(a, dev, s) : launch_phase_t<false, kMode | kStage>(a, dev, s);
+  return a.img_half ? launch_phase_t<true, kMode>(a, dev, s) : launch_phase_t<false, kMode>(a, dev, s);
 }
 // the method, or one of the ablations of Sec. 4 (a.ablation: bit 0 symmetric
 // propagation, bit 1 heuristic view selection)
-int launch_phase(const PhaseArgs& a, int n_sm, cudaStream_t s) {
-  if (a.tex_filter) return launch_phase_t<false, kTexture>(a, n_sm, s);
+int launch_phase(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
+  if (a.tex_filter) return launch_phase_t<false, kTexture>(a, dev, s);
   switch (a.ablation & 3) {
-    case kSymmetric: return launch_phase_m<kSymmetric>(a, n_sm, s);
-    case kHeuristic: return launch_phase_m<kHeuristic>(a, n_sm, s);
-    case kSymmetric | kHeuristic: return launch_phase_m<kSymmetric | kHeuristic>(a, n_sm, s);
-    default: return launch_phase_m<0>(a, n_sm, s);
+    case kSymmetric: return launch_phase_m<kSymmetric>(a, dev, s);
+    case kHeuristic: return launch_phase_m<kHeuristic>(a, dev, s);
+    case kSymmetric | kHeuristic: return launch_phase_m<kSymmetric | kHeuristic>(a, dev, s);
+    default: return launch_phase_m<0>(a, dev, s);
   }
 }
 

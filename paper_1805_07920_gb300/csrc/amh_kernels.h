@@ -3,13 +3,13 @@
 #include <cuda_runtime.h>
 
 #include "amh_device.cuh"
+#include "amh_launch.h"
 
 namespace amh {
-// random initialisation of every pixel on a device of n_sm multiprocessors;
-// returns a cudaError_t of the launch
-int launch_init(const PhaseArgs& a, int n_sm, cudaStream_t s);
+// random initialisation of every pixel; returns a cudaError_t of the launch
+int launch_init(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s);
 // one colour phase (a.color, a.t); returns a cudaError_t of the launch
-int launch_phase(const PhaseArgs& a, int n_sm, cudaStream_t s);
+int launch_phase(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s);
 // One state field (elem bytes per pixel: 16, 4 or 1) between the kernels'
 // layout (state_index) and a row-major W x H map in host or device memory.
 // Host maps go through a device buffer allocated and freed on the stream.

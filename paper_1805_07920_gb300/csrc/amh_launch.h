@@ -21,6 +21,20 @@ inline int blocks_per_sm(int64_t tiles, int n_sm, int most) {
   return (int)std::max<int64_t>(1, (tiles + rounds * n_sm - 1) / std::max<int64_t>(1, rounds * n_sm));
 }
 
+// The update through the texture unit's filter has so little arithmetic per
+// sample that the shared-memory reads of its window weights show where warps are
+// few.  With the weights in registers an SM takes `three` blocks instead of
+// `four`; that pays while it needs no more rounds for them, one or two.  Two
+// sources, four iterations, weights in shared memory (carve-out for the blocks
+// in use) / in registers / one kernel for all sizes before, in us: 320 x 240 394 /
+// 381 / 407, 360 x 270 505 / 488 / 509, 440 x 330 (one round or two) 635 / 830 / 636,
+// 520 x 390 960 / 939 / 1013, 640 x 480 (two or three) 1287 / 1363 / 1287.
+inline bool registers_pay(int64_t tiles, int n_sm, int three, int four) {
+  const int64_t r3 = (tiles + (int64_t)three * n_sm - 1) / ((int64_t)three * n_sm);
+  const int64_t r4 = (tiles + (int64_t)four * n_sm - 1) / ((int64_t)four * n_sm);
+  return r3 <= r4 && r3 <= 2;
+}
+
 // The shared-memory carve-out that holds `blocks` blocks of `smem` bytes (and the
 // 1 KB each that the system keeps), as a percentage; the rest of the unified L1
 // is texture and local-memory cache.  Rounded down: the device has a few sizes

@@ -9,12 +9,15 @@
 // neighbouring windows of the same source view.  Every (hypothesis, view)
 // loop runs with a warp-uniform view index (uniform texture handle).  The 36
 // bilateral weights of a pixel sit in shared memory (72 floats read once per
-// evaluation, conflict-free 16-byte loads): in registers they held the kernel
-// at 168 registers and 12 warps per SM, here 128 and 16.  The cost matrix and
-// the view weights are in local memory (L1).
+// evaluation, conflict-free 16-byte loads): in registers they hold the kernel
+// at 168 registers and 12 warps per SM, here 128 and 16 (kRegs is the form with
+// registers, kept where it is faster).  The cost matrix and the view weights
+// are in local memory (L1).
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "amh_device.cuh"
 
@@ -61,14 +64,33 @@ static_assert(acp_other_colour(), "propagation candidates lie on the other colou
 // packed moment updates: (w, w', w r, w' r') of pair m at q[m * kStep], kStep
 // pixels side by side.
 constexpr int kWinPairs = kWinS / 2;
+constexpr int kRowGroup = 3;              // see ncc_window
 template <int kStep>
 struct RefWin {
+  static constexpr int kRows = kRowGroup; // window rows in flight
   float4* q;
   float inv_sw, sum_wr, var_r;
+  __device__ __forceinline__ void put(int m, float w0, float w1, float wr0, float wr1) {
+    q[m * kStep] = make_float4(w0, w1, wr0, wr1);
+  }
   __device__ __forceinline__ void pair(int m, f2& w, f2& wr) const {
     const float4 v = q[m * kStep];
     w = pack2(v.x, v.y);
     wr = pack2(v.z, v.w);
+  }
+};
+// The same in registers: everything unrolled.
+struct RegWin {
+  static constexpr int kRows = kWinN;
+  f2 w2[kWinPairs], wr2[kWinPairs];
+  float inv_sw, sum_wr, var_r;
+  __device__ __forceinline__ void put(int m, float w0, float w1, float wr0, float wr1) {
+    w2[m] = pack2(w0, w1);
+    wr2[m] = pack2(wr0, wr1);
+  }
+  __device__ __forceinline__ void pair(int m, f2& w, f2& wr) const {
+    w = w2[m];
+    wr = wr2[m];
   }
 };
 constexpr int kBlockPixels = 128;         // pixels of a block, one per thread
@@ -93,8 +115,8 @@ __device__ __forceinline__ float ref_at(const A& a, size_t i) {
 template <bool kHalf>
 __host__ __device__ constexpr float tex_scale() { return kHalf ? 1.f : 255.f; }
 
-template <bool kHalf, int kStep, class A>
-__device__ __forceinline__ void load_ref_window(const A& a, int x, int y, RefWin<kStep>& rw) {
+template <bool kHalf, class A, class Win>
+__device__ __forceinline__ void load_ref_window(const A& a, int x, int y, Win& rw) {
   const float Ic = ref_at<kHalf, A>(a, (size_t)y * a.W + x);
   // w = exp(-e) relative to the largest weight: the statistics of Eq. (8) are
   // ratios of weighted sums, so the common factor cancels, and no weight
@@ -133,9 +155,7 @@ __device__ __forceinline__ void load_ref_window(const A& a, int x, int y, RefWin
     s2 = fmaf(wr, rc, s2);
   }
 #pragma unroll
-  for (int m = 0; m < kWinS / 2; m++) {
-    rw.q[m * kStep] = make_float4(wv[2 * m], wv[2 * m + 1], wrv[2 * m], wrv[2 * m + 1]);
-  }
+  for (int m = 0; m < kWinPairs; m++) rw.put(m, wv[2 * m], wv[2 * m + 1], wrv[2 * m], wrv[2 * m + 1]);
   rw.inv_sw = inv;
   rw.sum_wr = swr;
   rw.var_r = s2 * inv - (swr * inv) * (swr * inv);
@@ -277,7 +297,6 @@ struct RowFetch {
 // the first is used (about 110 of the 128 registers).  1600 x 1056, 10 sources,
 // five iterations with the proposal: 6 rows unrolled 33.5 ms, 3: 31.9, 2: 33.0
 // (12 warps per SM, weights in registers, everything unrolled: 38.0 before).
-constexpr int kRowGroup = 3;
 static_assert(kWinN % kRowGroup == 0, "the rows of a window are processed in whole groups");
 template <bool kHalf, int kFetch, class Win>
 __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& G, const Win& rw,
@@ -375,12 +394,12 @@ __device__ __forceinline__ float ncc_window(const ViewConst& V, const PairGeom& 
     }
   };
 #pragma unroll 1
-  for (int r0 = 0; r0 < kWinN; r0 += kRowGroup) {
-    RowFetch F[kRowGroup];
+  for (int r0 = 0; r0 < kWinN; r0 += Win::kRows) {
+    RowFetch F[Win::kRows];
 #pragma unroll
-    for (int u = 0; u < kRowGroup; u++) issue((float)(r0 + u), F[u]);
+    for (int u = 0; u < Win::kRows; u++) issue((float)(r0 + u), F[u]);
 #pragma unroll
-    for (int u = 0; u < kRowGroup; u++) consume(r0 + u, F[u]);
+    for (int u = 0; u < Win::kRows; u++) consume(r0 + u, F[u]);
   }
   float m1a, m1b, m2a, m2b, mra, mrb;
   unpack2(acc1, m1a, m1b);
@@ -688,6 +707,9 @@ constexpr int kTexture = 4;
 // kStage: the 8 x N matrix sweep stages shared-memory sample boxes (the whole
 // block calls update_pixel together, pixels outside the image included)
 constexpr int kStage = 8;
+// kRegs -- the window weights in registers, three blocks per SM, and no help in
+// the refinement (a helper reads the other lane's weights).
+constexpr int kRegs = 16;
 
 // ---------------------------------------------------------------------------
 // one pixel's checkerboard update.  All lanes of the warp call it; one whose
@@ -699,6 +721,7 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
                                              int* npairs, float4* win, uint8_t* slots, bool live, StageShared* ss = nullptr) {
   constexpr bool kTex = (kMode & kTexture) != 0;
   constexpr bool kStaged = (kMode & kStage) != 0;
+  constexpr bool kRegWin = (kMode & kRegs) != 0;
   static_assert(!(kStaged && kTex), "the staged sweep gathers; the texture-filter form does not stage");
   const int N = a.N;
   // the pixel's state index (32-bit: a state holds fewer than 2^31 entries)
@@ -761,8 +784,8 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
     valid |= 1u << g;
   }
 
-  PixelWin rw;
-  rw.q = win;
+  typename std::conditional<kRegWin, RegWin, PixelWin>::type rw;
+  if constexpr (!kRegWin) rw.q = win;
   if (live) load_ref_window<kHalf>(a, x, y, rw);
 
   // --- Eq. (1): the 8 x N cost matrix (views outer: the 8 hypotheses of a view
@@ -928,69 +951,79 @@ __device__ __forceinline__ void update_pixel(const A& a, PixelArrays& sm, int x,
   for (int j = 0; j < N; j++) {
     const float wj = sm.wt(j);
     uint32_t todo = wj > 0.f ? cand_live : 0u;
-    // Each turn a lane takes one of its candidates; a lane with none left takes
-    // a second one of a lane that has more (its plane, ray and window by
-    // shuffles; the weights are in shared memory) and hands the cost back.  At
-    // t >= 3 the candidates took 24 % of the gathers for 13 % more evaluations
-    // (about half the lanes idle); with the help 15 %.  3200 x 2112, 10 sources,
-    // six iterations 159 -> 154 ms, learned form at 1600 x 1056 33.5 -> 32.8.
-    while (__any_sync(0xffffffffu, todo != 0u)) {
-      const int ci = todo ? __ffs(todo) - 1 : -1;
-      todo &= todo - 1u;                                   // 0 stays 0
-      const uint32_t idle = __ballot_sync(0xffffffffu, ci < 0), more = __ballot_sync(0xffffffffu, todo != 0u);
-      const uint32_t below = (1u << lane) - 1u;
-      const int pairs = min(__popc(idle), __popc(more));
-      float4 c2 = ci >= 0 ? sm.cc(ci) : make_float4(0.f, 0.f, 0.f, 0.f);
-      bool ok2 = ci >= 0 && ((okm >> ci) & 1u);
-      float3 ray2 = ray;
-      PixelWin rw2 = rw;
-      int cj = -1, partner = lane;
-      if (pairs > 0) {                                     // the same for every lane
-        const int rank = __popc((ci < 0 ? idle : more) & below);
-        const bool helps = ci < 0 && rank < pairs, helped = todo != 0u && rank < pairs;
-        // the r-th idle lane and the r-th lane with more meet over the warp's
-        // slots: slot[r] the helped lane, slot[32 + r] the helper
-        if (helped) slots[rank] = (uint8_t)lane;
-        if (helps) slots[32 + rank] = (uint8_t)lane;
-        __syncwarp();
-        if (helps) partner = slots[rank];
-        if (helped) {
-          partner = slots[32 + rank];
-          cj = __ffs(todo) - 1;
-          todo &= todo - 1u;
-        }
-        __syncwarp();
-        const float4 cs = cj >= 0 ? sm.cc(cj) : c2;
-        const int oks = cj >= 0 ? (int)((okm >> cj) & 1u) : 0;
-        const float4 cr = make_float4(__shfl_sync(0xffffffffu, cs.x, partner), __shfl_sync(0xffffffffu, cs.y, partner), 0.f,
-                                      __shfl_sync(0xffffffffu, cs.w, partner));
-        const int okr = __shfl_sync(0xffffffffu, oks, partner);
-        const float rx = __shfl_sync(0xffffffffu, ray.x, partner), ry = __shfl_sync(0xffffffffu, ray.y, partner),
-                    rz = __shfl_sync(0xffffffffu, ray.z, partner);
-        const float i2 = __shfl_sync(0xffffffffu, rw.inv_sw, partner), s2 = __shfl_sync(0xffffffffu, rw.sum_wr, partner),
-                    v2 = __shfl_sync(0xffffffffu, rw.var_r, partner);
-        if (helps) {
-          c2 = cr;
-          ok2 = okr != 0;
-          ray2 = make_float3(rx, ry, rz);
-          rw2.q = rw.q + (partner - lane);
-          rw2.inv_sw = i2;
-          rw2.sum_wr = s2;
-          rw2.var_r = v2;
-        }
+    if constexpr (kRegWin) {
+      while (todo) {
+        const int ci = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const float m = fmaf(wj, ncc_cost<kHalf, kTex>(a.v[j], sm.cc(ci), (okm >> ci) & 1u, ray, rw, npairs), sm.m(0, ci, N));
+        sm.m(0, ci, N) = m;
+        if (!(m * inv_sw < bm)) cand_live &= ~(1u << ci);
       }
-      float m = kWorst;
-      if (ci >= 0 || partner != lane) m = ncc_cost<kHalf, kTex>(a.v[j], c2, ok2, ray2, rw2, npairs);
-      const float mj = pairs > 0 ? __shfl_sync(0xffffffffu, m, partner) : 0.f;
-      if (ci >= 0) {
-        const float t = fmaf(wj, m, sm.m(0, ci, N));
-        sm.m(0, ci, N) = t;
-        if (!(t * inv_sw < bm)) cand_live &= ~(1u << ci);
-      }
-      if (cj >= 0) {
-        const float t = fmaf(wj, mj, sm.m(0, cj, N));
-        sm.m(0, cj, N) = t;
-        if (!(t * inv_sw < bm)) cand_live &= ~(1u << cj);
+    } else {
+      // Each turn a lane takes one of its candidates; a lane with none left takes
+      // a second one of a lane that has more (its plane, ray and window by
+      // shuffles; the weights are in shared memory) and hands the cost back.  At
+      // t >= 3 the candidates took 24 % of the gathers for 13 % more evaluations
+      // (about half the lanes idle); with the help 15 %.  3200 x 2112, 10 sources,
+      // six iterations 159 -> 154 ms, learned form at 1600 x 1056 33.5 -> 32.8.
+      while (__any_sync(0xffffffffu, todo != 0u)) {
+        const int ci = todo ? __ffs(todo) - 1 : -1;
+        todo &= todo - 1u;                                   // 0 stays 0
+        const uint32_t idle = __ballot_sync(0xffffffffu, ci < 0), more = __ballot_sync(0xffffffffu, todo != 0u);
+        const uint32_t below = (1u << lane) - 1u;
+        const int pairs = min(__popc(idle), __popc(more));
+        float4 c2 = ci >= 0 ? sm.cc(ci) : make_float4(0.f, 0.f, 0.f, 0.f);
+        bool ok2 = ci >= 0 && ((okm >> ci) & 1u);
+        float3 ray2 = ray;
+        PixelWin rw2 = rw;
+        int cj = -1, partner = lane;
+        if (pairs > 0) {                                     // the same for every lane
+          const int rank = __popc((ci < 0 ? idle : more) & below);
+          const bool helps = ci < 0 && rank < pairs, helped = todo != 0u && rank < pairs;
+          // the r-th idle lane and the r-th lane with more meet over the warp's
+          // slots: slot[r] the helped lane, slot[32 + r] the helper
+          if (helped) slots[rank] = (uint8_t)lane;
+          if (helps) slots[32 + rank] = (uint8_t)lane;
+          __syncwarp();
+          if (helps) partner = slots[rank];
+          if (helped) {
+            partner = slots[32 + rank];
+            cj = __ffs(todo) - 1;
+            todo &= todo - 1u;
+          }
+          __syncwarp();
+          const float4 cs = cj >= 0 ? sm.cc(cj) : c2;
+          const int oks = cj >= 0 ? (int)((okm >> cj) & 1u) : 0;
+          const float4 cr = make_float4(__shfl_sync(0xffffffffu, cs.x, partner), __shfl_sync(0xffffffffu, cs.y, partner), 0.f,
+                                        __shfl_sync(0xffffffffu, cs.w, partner));
+          const int okr = __shfl_sync(0xffffffffu, oks, partner);
+          const float rx = __shfl_sync(0xffffffffu, ray.x, partner), ry = __shfl_sync(0xffffffffu, ray.y, partner),
+                      rz = __shfl_sync(0xffffffffu, ray.z, partner);
+          const float i2 = __shfl_sync(0xffffffffu, rw.inv_sw, partner), s2 = __shfl_sync(0xffffffffu, rw.sum_wr, partner),
+                      v2 = __shfl_sync(0xffffffffu, rw.var_r, partner);
+          if (helps) {
+            c2 = cr;
+            ok2 = okr != 0;
+            ray2 = make_float3(rx, ry, rz);
+            rw2.q = rw.q + (partner - lane);
+            rw2.inv_sw = i2;
+            rw2.sum_wr = s2;
+            rw2.var_r = v2;
+          }
+        }
+        float m = kWorst;
+        if (ci >= 0 || partner != lane) m = ncc_cost<kHalf, kTex>(a.v[j], c2, ok2, ray2, rw2, npairs);
+        const float mj = pairs > 0 ? __shfl_sync(0xffffffffu, m, partner) : 0.f;
+        if (ci >= 0) {
+          const float t = fmaf(wj, m, sm.m(0, ci, N));
+          sm.m(0, ci, N) = t;
+          if (!(t * inv_sw < bm)) cand_live &= ~(1u << ci);
+        }
+        if (cj >= 0) {
+          const float t = fmaf(wj, mj, sm.m(0, cj, N));
+          sm.m(0, cj, N) = t;
+          if (!(t * inv_sw < bm)) cand_live &= ~(1u << cj);
+        }
       }
     }
   }

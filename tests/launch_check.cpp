@@ -30,6 +30,13 @@ int main() {
         // fewer tiles than SMs: one block per tile
         CHECK(tiles > sm || (k == 1 && grid == tiles), "sm %d most %d tiles %ld", sm, most, (long)tiles);
       }
+  // window weights in registers: never more rounds at three blocks than at four, at most two
+  for (int sm : {1, 78, 152})
+    for (int64_t tiles = 1; tiles < 3000; tiles++, n++) {
+      const bool r = registers_pay(tiles, sm, 3, 4);
+      const int64_t r3 = (tiles + 3 * sm - 1) / (3 * sm), r4 = (tiles + 4 * sm - 1) / (4 * sm);
+      CHECK(r == (r3 <= 2 && r3 == r4), "sm %d tiles %ld", sm, (long)tiles);
+    }
   // the carve-out holds the blocks in the sizes the device offers (it takes the next one up)
   const int sizes[] = {0, 8, 16, 32, 64, 100, 132, 164, 196, 228}, smem_sm = 228 * 1024;
   for (int smem : {SMEM})

@@ -15,7 +15,8 @@ def test_launch_arithmetic(tmp_path):
     gxx = shutil.which("g++")
     if gxx is None:
         pytest.skip("g++ not available")
-    smem = {v["smem"] for k, v in _reports().items() if "batch_phase_kernel" in k or "batch_init_kernel" in k}
+    kernels = ("batch_phase_kernel", "batch_init_kernel", "12phase_kernel", "11init_kernel")     # one thread per pixel
+    smem = {v["smem"] for k, v in _reports().items() if any(n in k for n in kernels) and v["smem"]}
     assert smem and min(smem) > 0
     exe = str(tmp_path / "launch_check")
     subprocess.run([gxx, "-std=c++17", "-O1", "-DSMEM=" + ",".join(map(str, sorted(smem))), "-o", exe,

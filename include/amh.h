@@ -447,9 +447,20 @@ AMH_API int amh_gather_peak(double* samples_per_s);
 AMH_API int amh_get_info(const amh_ctx* ctx, int32_t* width, int32_t* height,
                          int32_t* n_src, int32_t* t);
 
+/* Warps that share 32 pixels of a width x height reference with n_src sources on
+ * a device of n_sm multiprocessors: 16, 8 or 4 where the image is too small to
+ * fill the device with one thread per pixel, else 1; of the initialisation and
+ * of a colour phase (either may be NULL).  The ablations, the staged sweep and
+ * the batch always take 1.  The results are the same bits.  Host arithmetic. */
+AMH_API int amh_update_warps(int32_t width, int32_t height, int32_t n_src, int32_t n_sm, int32_t* init, int32_t* phase);
+
 /* Number of (hypothesis, view) cost evaluations the kernels have performed
  * since the last reset (each is one 36-sample warped bilateral NCC).  The
- * count is kept on the device; reading it synchronises the stream. */
+ * count is kept on the device; reading it synchronises the stream.  It is of
+ * the work done, not of the result: where warps share the pixels
+ * (amh_update_warps), a phase with one or two refinement candidates (t < 3)
+ * evaluates each on every view of nonzero weight, while one thread per pixel
+ * drops a candidate once it cannot win, so that such an image counts more. */
 AMH_API int amh_pair_count(amh_ctx* ctx, uint64_t* count, int32_t reset);
 /* The same count (total, may be NULL) and, of those, the evaluations whose 36
  * samples were read from a shared-memory box instead of the texture unit

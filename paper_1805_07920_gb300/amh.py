@@ -29,7 +29,7 @@ BATCH_VARIANTS = 5                   # AMH_BATCH_VARIANTS: tile / warp-layout va
 
 EXPORTS = ["amh_default_params", "amh_create", "amh_set_stream", "amh_init_random",
            "amh_step_phase", "amh_iterate", "amh_get_state", "amh_set_state", "amh_read_maps",
-           "amh_get_info", "amh_pair_count", "amh_pair_counts", "amh_synchronize", "amh_last_error", "amh_destroy",
+           "amh_get_info", "amh_update_warps", "amh_pair_count", "amh_pair_counts", "amh_synchronize", "amh_last_error", "amh_destroy",
            "amh_read_maps_noalloc", "amh_batch_create", "amh_batch_init_random", "amh_batch_step_phase",
            "amh_batch_iterate", "amh_batch_run", "amh_batch_set_variant", "amh_batch_autotune",
            "amh_batch_info", "amh_batch_get_state", "amh_batch_pair_count", "amh_batch_synchronize",
@@ -175,6 +175,18 @@ def default_params(**kw) -> Params:
     for k, v in kw.items():
         setattr(p, k, v)
     return p
+
+
+def update_warps(width: int, height: int, n_src: int, n_sm: int) -> tuple[int, int]:
+    """(initialisation, colour phase) warps that share 32 pixels of such a
+    reference on a device of n_sm multiprocessors (``amh_update_warps``)."""
+    L = lib()
+    L.amh_update_warps.argtypes = [_i32, _i32, _i32, _i32, ctypes.POINTER(_i32), ctypes.POINTER(_i32)]
+    a, b = _i32(), _i32()
+    rc = L.amh_update_warps(int(width), int(height), int(n_src), int(n_sm), ctypes.byref(a), ctypes.byref(b))
+    if rc != AMH_OK:
+        raise AmhError(rc, L.amh_last_error(None).decode())
+    return a.value, b.value
 
 
 def make_cameras(cams) -> ctypes.Array:

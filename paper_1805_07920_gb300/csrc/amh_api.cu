@@ -514,6 +514,14 @@ AMH_API int amh_get_info(const amh_ctx* c, int32_t* w, int32_t* h, int32_t* n, i
   return AMH_OK;
 }
 
+AMH_API int amh_update_warps(int32_t width, int32_t height, int32_t n_src, int32_t n_sm, int32_t* init, int32_t* phase) {
+  if (width < 1 || height < 1 || n_src < 1 || n_src > AMH_MAX_SRC || n_sm < 1)
+    return fail_no_context(AMH_EINVAL, "amh_update_warps: sizes out of range");
+  if (init) *init = team_warps(init_groups(width, height), n_src, n_sm, true);
+  if (phase) *phase = team_warps(phase_groups(width, height), n_src, n_sm, false);
+  return AMH_OK;
+}
+
 AMH_API int amh_pair_counts(amh_ctx* c, uint64_t* total, uint64_t* staged, int32_t reset) {
   if (!c) return AMH_EINVAL;
   unsigned long long v[2 * kPairCounters];

@@ -124,23 +124,6 @@ int launch_blocks(K kernel, dim3 grid, int most, int smem, int dynamic, const Ph
   return (int)cudaGetLastError();
 }
 
-// Warps per 32 pixels for a launch over `groups` groups of 32 pixels: 16, 8 or 4
-// (a team), or 1 (one thread per pixel).  A team's fixed work (propagation,
-// window, view selection, barriers) is repeated or waited for by its warps, so
-// it pays while the GPU has room for it: 16 or 8 warps while all teams fit at
-// once with 16 warps per SM, 4 up to 0.8 of the warps that one thread per pixel
-// can keep resident (0.4 with fewer than four views, where the fixed work
-// weighs more).  Six sources, four iterations, 1 / 4 / 8 / 16 warps in us:
-// 64x48 750 / 328 / 233 / 229, 160x120 802 / 385 / 324 / 414, 320x240 1143 /
-// 1018 / 1078 / 1474, 400x300 1683 / 1563 / 1635 / 2299, 440x330 1748 / 1880 /
-// 1951 / 2794; with two sources 320x240 takes 462 / 501 / 611 / 972 (each phase
-// set up after the one before had ended, see launch_phase_team).
-int team_warps(int groups, int n_src, int n_sm) {
-  const int warps = 16 * n_sm;
-  if (groups * 16 <= warps) return 16;
-  if (groups * 8 <= warps) return 8;
-  return groups * 10 <= warps * (n_src < 4 ? 4 : 8) ? 4 : 1;
-}
 // Static and dynamic shared memory together go past the default limit of 48 KB:
 // the team kernels' with many views, the staged sweep's boxes beside the window
 // weights.  Allowed once per device.
@@ -182,7 +165,7 @@ int launch_phase_team(const PhaseArgs& a, cudaStream_t s) {
 
 template <bool kHalf, bool kTex>
 int launch_init_t(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
-  switch (team_warps(((a.W + 7) / 8) * ((a.H + 3) / 4), a.N, dev.n_sm)) {
+  switch (team_warps(init_groups(a.W, a.H), a.N, dev.n_sm, true)) {
     case 16: return launch_init_team<kHalf, kTex, 16>(a, s);
     case 8: return launch_init_team<kHalf, kTex, 8>(a, s);
     case 4: return launch_init_team<kHalf, kTex, 4>(a, s);
@@ -201,7 +184,7 @@ int launch_init(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
 template <bool kHalf, int kMode>
 int launch_phase_t(const PhaseArgs& a, const DeviceShape& dev, cudaStream_t s) {
   if constexpr (kMode == 0 || kMode == kTexture) {   // the ablations and the staged sweep: one thread per pixel
-    switch (team_warps(((a.W + 15) / 16) * ((a.H + 3) / 4), a.N, dev.n_sm)) {
+    switch (team_warps(phase_groups(a.W, a.H), a.N, dev.n_sm, false)) {
       case 16: return launch_phase_team<kHalf, kMode == kTexture, 16>(a, s);
       case 8: return launch_phase_team<kHalf, kMode == kTexture, 8>(a, s);
       case 4: return launch_phase_team<kHalf, kMode == kTexture, 4>(a, s);

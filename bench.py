@@ -60,7 +60,7 @@ KNOWN_TRAFFIC: dict[str, float] = {
 }
 
 
-PHASE_KERNEL_SOURCES = ("amh_device.cuh", "amh_kernels.cu", "amh_kernels.h", "amh_update.cuh")
+PHASE_KERNEL_SOURCES = ("amh_device.cuh", "amh_kernels.cu", "amh_kernels.h", "amh_launch.h", "amh_update.cuh")
 # the batched form's variants (AMH_BATCH_VARIANTS): block tile / warp pixel layout
 VARIANT_NAMES = ["16x16/warp 16x4", "32x8/warp 32x2", "64x4/warp 64x1", "16x16/warp 8x8", "32x8/warp 16x4"]
 

@@ -34,7 +34,10 @@ namespace {
 using namespace upd;
 
 constexpr int kBThreads = 128;
-constexpr int kBBlocksPerSM = 4;          // as the single contexts' phase kernel
+// As the single contexts' phase kernel.  The item's constants in shared memory
+// instead of kernel arguments cost the uint8 and FP16 forms a spill of 20 bytes
+// of stores and 44 of loads.
+constexpr int kBBlocksPerSM = 4;
 constexpr int kMaxRefs = 256;
 constexpr int kViewWords = (int)(sizeof(ViewConst) / sizeof(float));   // a view table entry in 4-byte words
 static_assert(sizeof(ViewConst) % sizeof(float) == 0, "view table entries are whole words");

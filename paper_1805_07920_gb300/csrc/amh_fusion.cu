@@ -60,7 +60,7 @@ __device__ __noinline__ float median16_sorted(const float* __restrict__ in, int 
 // (9 comparators); then the 8th and 9th smallest of the 16 are max_i min(A_i,
 // B_7-i) and min_i max(A_i, B_7-i).  About 56 min / max per output instead of
 // the 240 of a sort of its own, which bound it (3200 x 2112: 102 us before,
-// 29 us now; reading and writing the map once takes 8).  A warp whose columns
+// 31 us now; reading and writing the map once takes 8).  A warp whose columns
 // hold a NaN sorts each window in full: with a NaN the result depends on the
 // order of the comparisons.
 constexpr int kMedRows = 16, kMedCols = 29, kMedWarps = 4;
@@ -158,17 +158,17 @@ constexpr float kTiny = 1e-30f, kHuge = 1e30f;
 
 // A block takes 32 x 16 pixels of one view, a warp 32 pixels of a row;
 // neighbouring blocks take the same tile of all views, so that what they gather
-// from the other views is in L2 (view after view, ten 1600 x 1056 views took
-// 1384 us instead of 1171).  What bounds it: instruction issue, about 200 per
-// agreeing check of which 130 are the rounded arithmetic, then the gathers.
-// Before, per view pair five correctly rounded divisions and three roots with
-// their branches, the views' constants by indexed loads, a 64-bit division per
-// pixel and 24-byte strided stores: ten 1600 x 1056 views 1670 us, now 1017; twenty
-// views around a ring, where most checks fail, 8.5 ms, now 7.1 ms.  With four
-// rows instead of 16 per block the set-up of the constants shows: 1116 us and 10.3
-// ms.  Measured and left: two or four pixels per thread 1566 / 1827 us
-// (registers), the next view's fetches issued ahead 1289, five blocks of 8 warps
-// (48 registers) 1322.  Points leave through shared memory as rows of 768 bytes.
+// from the other views is in L2.  What bounds it: instruction issue, about 200
+// per check and warp, then the gathers.  Ten 1600 x 1056 views take 1007 us,
+// twenty views around a ring, where most checks fail, 7.1 ms; with five correctly
+// rounded divisions and three roots per check and their branches, the views'
+// constants by indexed loads, a 64-bit division per pixel and 24-byte strided
+// stores 1790 us and 8.5 ms.  On the way, with four rows per block instead of 16
+// (the set-up of the constants shows: 1116 us, 10.3 ms): one view after another
+// 1384 us where tile after tile took 1171; two or four pixels per thread 1566 /
+// 1827 (registers), the next view's fetches issued ahead 1289, five blocks of 8
+// warps (48 registers) 1322.  Points leave through shared memory as rows of 768
+// bytes.
 constexpr int kFuseWarps = 4, kFuseRows = 4 * kFuseWarps, kFuseBlocksPerSM = 8;   // 64 registers
 // a view's constants in shared memory, read as float4
 struct FuseShared {

@@ -18,7 +18,7 @@ using namespace upd;
 constexpr int kTile = 16;
 constexpr int kThreads = 128;
 // 128 registers per thread; the window weights are 36 KB of shared memory per
-// block, so 4 blocks leave about 100 KB of L1.  Five blocks (96 registers): the
+// block, so 4 blocks leave 92 KB of L1.  Five blocks (96 registers): the
 // learned form at 1600 x 1056 32.2 ms against 31.9, 640 x 480 3.99 against 3.65.
 // The staged sweep's boxes and the window weights in registers (168) allow 3.
 constexpr int kPhaseBlocksPerSM = 4, kThreeBlocksPerSM = 3;

@@ -558,8 +558,8 @@ __device__ __forceinline__ float4 refine_candidate(const A& a, int x, int y, flo
 
 // Per-pixel working arrays of one thread (local memory, cached in L1): the
 // 8 x N cost matrix of Eq. (1), the N view weights and the 8 propagated planes
-// as (c = K^-T n / d, 1 / D).  Shared memory stays unused so that L1 serves the texture
-// gathers.
+// as (c = K^-T n / d, 1 / D).  Shared memory holds the window weights only; the
+// rest of the unified L1 is for these arrays and the texture gathers.
 struct PixelArrays {
   float M[kRegions * kMaxSrc];
   float w[kMaxSrc];
@@ -574,7 +574,7 @@ struct PixelArrays {
 // Eqs. (2)-(5) of one view, from its costs as they come (rows of invalid regions
 // are left out of the counts and of the mean of Eq. (4)): counted beside the
 // matrix, because a pass over the finished matrix read it back from the L2 (the
-// blocks of an SM hold 250 KB of local memory against about 100 KB of L1).
+// blocks of an SM hold 250 KB of local memory against 92 KB of L1).
 struct ViewScore {
   int good = 0, bad = 0;
   float psi = 0.f;

@@ -450,8 +450,9 @@ AMH_API int amh_get_info(const amh_ctx* ctx, int32_t* width, int32_t* height,
 /* Warps that share 32 pixels of a width x height reference with n_src sources on
  * a device of n_sm multiprocessors: 16, 8 or 4 where the image is too small to
  * fill the device with one thread per pixel, else 1; of the initialisation and
- * of a colour phase (either may be NULL).  The ablations, the staged sweep and
- * the batch always take 1.  The results are the same bits.  Host arithmetic. */
+ * of a colour phase (either may be NULL).  The phases of the ablations and of the
+ * staged sweep (t >= 1) take 1 whatever the size, and so does the batch.  The
+ * results are the same bits.  Host arithmetic. */
 AMH_API int amh_update_warps(int32_t width, int32_t height, int32_t n_src, int32_t n_sm, int32_t* init, int32_t* phase);
 
 /* Number of (hypothesis, view) cost evaluations the kernels have performed
